@@ -63,16 +63,16 @@ SUB_STEPS = {"single": 400, "orbit": 400, "ragged": 40, "recon": 30, "largek": 2
 # excluded) and MUFU operations (ex2, rcp, rsqrt), counted operation by operation
 # in docs/opcount.md from the formulas, with and without the normal plane.
 OPS = {  # normals -> (fwd FP32, fwd MUFU, bwd FP32, bwd MUFU), with pose gradients
-    True: (56, 4, 110, 4),
-    False: (35, 3, 63, 3),  # without normals the second projection of u is skipped (7 operations)
+    True: (36, 4, 88, 4),
+    False: (25, 3, 51, 3),
 }
-# The algorithmic minimum of the whitened formulation (docs/opcount.md): the
-# executed counts above less the operations of the compensated geometry (16 with
-# normals, 9 without) and the rsqrt guard of the normal.
-ALGO_OPS = {True: (39, 93), False: (26, 54)}  # normals -> (fwd FP32, bwd FP32), with pose gradients
-# Without pose gradients the two-parameter adjoint needs only the lower triangle of
-# sum v abar^T (6 of its 9 accumulations per pair).
-NO_POSE_SAVING = 3
+# The world-frame form of batches of at most WORLD_RAYS rays.
+OPS_WORLD = {True: (56, 4, 110, 4), False: (35, 3, 63, 3)}
+WORLD_RAYS = 131072
+# Operations that only the pose gradients need (of the camera-plane form: five sums
+# with the normal plane, nothing without; of the world-frame form: three sums).
+POSE_OPS = {True: 9, False: 0}
+POSE_OPS_WORLD = {True: 3, False: 3}
 # Alpha-compositing variant (Sec. 3.3): per pair, the same geometry plus the
 # transmittance and weight arithmetic (prefix sums, T = e^-S, 1 - e^-delta by its
 # series), and in the backward a re-render, the per-pair weight adjoint and the
@@ -132,7 +132,7 @@ def csrc_sha256() -> str:
 
     d = os.path.join(ROOT, "paper_2308_14737_gb300", "csrc")
     h = hashlib.sha256()
-    for name in ("fmb_backward.cu", "fmb_internal.cuh", "fmb_f32x2.cuh"):
+    for name in ("fmb_backward.cu", "fmb_cam.cuh", "fmb_internal.cuh", "fmb_f32x2.cuh"):
         h.update(name.encode())
         with open(os.path.join(d, name), "rb") as fh:
             h.update(fh.read())
@@ -471,9 +471,10 @@ def measure_workload(args, name, steps, warmup, dev, ws=1, extras=True, cpu=True
 
     clock_for_peak = 2070.0
     peak = peak_fp32_gops(clock_for_peak)
-    f32f, mf, f32b, mb = (OPS_AC if ac else OPS)[bool(wl["normals"])]
+    few = s.n_pixels <= WORLD_RAYS
+    f32f, mf, f32b, mb = (OPS_AC if ac else OPS_WORLD if few else OPS)[bool(wl["normals"])]
     if not ac and not want_pose:
-        f32b -= NO_POSE_SAVING
+        f32b -= (POSE_OPS_WORLD if few else POSE_OPS)[bool(wl["normals"])]
     roofline = {
         "bound": "alu",
         "kernel": ("backward_ac_kernel" if ac else "backward_kernel") + " (fmb_render_backward call)",
@@ -492,17 +493,6 @@ def measure_workload(args, name, steps, warmup, dev, ws=1, extras=True, cpu=True
         "step_frac": pairs * (f32f + f32b) / (ms_step * 1e-3) / 1e9 / peak,
     }
     roofline["frac"] = roofline["achieved"] / roofline["peak"]
-    if not ac:
-        # the same times against the method's own operations only (the compensated
-        # geometry's extra operations left out of the count)
-        cf, cb = ALGO_OPS[bool(wl["normals"])]
-        if not want_pose:
-            cb -= NO_POSE_SAVING
-        roofline["method_ops_only"] = {
-            "bwd_fp32": cb, "fwd_fp32": cf,
-            "frac": pairs * cb / (bwd_ms * 1e-3) / 1e9 / peak,
-            "forward_frac": pairs * cf / (fwd_ms * 1e-3) / 1e9 / peak,
-            "step_frac": pairs * (cf + cb) / (ms_step * 1e-3) / 1e9 / peak}
     # the committed ncu summaries cover the two-parameter backward on the orbit and large-K workloads
     roofline["traffic"] = (profiled_traffic({k: int(getattr(tuned_params, k)) for k in autotune.TUNED_FIELDS},
                                             workload=name)

@@ -4,7 +4,8 @@
 //
 //   [0, 256)            status word (int) at 0, forward work counter at 64,
 //                       backward work counter at 128
-//   [256, 256 + 64 R)   R per-(view, Gaussian) records, R = sum over views of K
+//   [256, 256 + 64 R)   R per-(view, Gaussian) records, R = sum over views of K, each
+//                       view's K rounded up to an even count
 //   [.., ..)            backward partials (deterministic mode only)
 #include <algorithm>
 #include <cmath>
@@ -36,6 +37,16 @@ constexpr size_t kHeaderBytes = 256;
 constexpr size_t kFwdCounterOffset = 64;
 constexpr size_t kBwdCounterOffset = 128;
 constexpr int kDefaultRpt = 2;
+// Two-parameter calls of at most this many rays (and the stored-intermediate mode) run
+// in the world-frame form, larger ones in the camera-plane form, which needs 0.64-0.82
+// of the operations.  Both have the same error against FP64 on average, but not the same
+// rounding: over 12 scenes the ratio of their gradient errors spreads by a factor of
+// 1.3-1.7 for one view of 9 000 to 120 000 rays, where single rays show in the sums, and
+// by 1.2 from 300 000 rays on.  Small calls have little to gain: they are bound by
+// latency and launches (64x64 view at K = 40, forward and backward replayed: 41.5 us
+// world, 38.1 camera; 50 000-ray minibatch at K = 256, eager calls: 167 and 166 us),
+// while 150 000 rays at K = 100-4096 already gain 1.2-1.35x.
+constexpr long long kWorldRays = 131072;
 constexpr int kMaxGaussPerCta = 256;
 constexpr long long kMaxK = 1 << 22;
 constexpr int kMaxKAlphaCompositing = 256;
@@ -76,9 +87,9 @@ static double bwd_lane_fill(int K, int T, int n) {
 // 100 (3 subgroups of 50 threads) instead of one of 200 (one subgroup of 100).
 // min_blocks > 0 (the bwd_gblocks hint) raises the count to at least that many,
 // for batches too small to fill the GPU with one block per ray tile.  even_blocks
-// (the stored-intermediate adjoint, which reads a thread's two Gaussians' stored
-// values with one 8-byte load) rounds the block size up to an even count, so that
-// every block starts at an even Gaussian index.
+// (the render's adjoint: records and stored pair values hold two Gaussians) rounds
+// the block size up to an even count, so that every block starts at an even Gaussian
+// index.
 BwdBlocking bwd_blocking(int K, int T, int min_blocks = 0, bool even_blocks = false) {
   const int gbmax = std::min(2 * T, kMaxGaussPerCta);
   const int n_min = (K + gbmax - 1) / gbmax;
@@ -136,11 +147,13 @@ struct Plan {
   std::vector<fmb::Batch> fwd;  // forward launches (tiles of rays)
   std::vector<fmb::Batch> bwd;  // backward launches (ray tiles x Gaussian blocks)
   std::vector<fmb::BigBatch> fwd_big, bwd_big, fmerge_big;
-  long long n_records = 0;
+  long long n_records = 0;  // record slots (each view's Gaussians, rounded up to an even count)
+  long long n_pairs = 0;    // sum over views of K
   long long part_floats = 0;
   long long pair_stride = 0;  // stored-intermediate mode: floats per per-pair array
   long long n_gauss = 0;
   int maxK = 0;
+  bool world = false;  // the two-parameter kernels in the world-frame form (fmb_world_*.cu)
   int rpt = kDefaultRpt;
   int ray_tile = 480;
   int bwd_threads = 160;
@@ -239,6 +252,18 @@ void order_items(B& b, Cost cost, Count count) {
   b.n_items = static_cast<int>(acc);
 }
 
+// Blocks of an even size: the camera-plane records and the stored pair values hold two
+// Gaussians.
+bool even_blocks(const fmb_params* p, const Plan& pl) {
+  return p->variant == 0 && (!pl.world || p->store_pairs != 0);
+}
+
+long long total_entries(const fmb_view* views, int n_views) {
+  long long n = 0;
+  for (int i = 0; i < n_views; ++i) n += view_entries(views[i]);
+  return n;
+}
+
 // The views in batches of up to B::kCapacity, one batch per launch: each view's
 // per-launch record (forward and backward tiling), the running offsets of its
 // records, partial slots and stored pairs, and the batch's work items in cost order.
@@ -270,10 +295,11 @@ void fill_batches(Plan& pl, const fmb_params* p, const long long* offs, int n_vi
       d.K = static_cast<int>(offs[v.object + 1] - offs[v.object]);
       pl.maxK = std::max(pl.maxK, d.K);
       d.gauss_off = static_cast<int>(offs[v.object]);
-      if (rec + d.K > kMaxRecords) throw std::runtime_error("too many (view, Gaussian) pairs in one batch");
+      if (pl.n_pairs + d.K > kMaxRecords) throw std::runtime_error("too many (view, Gaussian) pairs in one batch");
+      pl.n_pairs += d.K;
       d.rec_off = static_cast<int>(rec);
       d.pix_off = v.pix_offset;
-      rec += d.K;
+      rec += (d.K + 1) & ~1;  // the render's records hold two Gaussians (fmb_cam.cuh)
       const long long P = view_entries(v);
       pl.n_entries += P;
       d.rays = v.rays;
@@ -288,6 +314,7 @@ void fill_batches(Plan& pl, const fmb_params* p, const long long* offs, int n_vi
         // split s renders Gaussians [s GB, min(K, (s + 1) GB)); every split is non-empty
         const int S0 = std::min(pl.ksplit, d.K);
         df.GB = (d.K + S0 - 1) / S0;
+        if (!ac && !pl.world && S0 > 1) df.GB = (df.GB + 1) & ~1;  // whole records of two Gaussians
         df.n_gblocks = (d.K + df.GB - 1) / df.GB;
         df.S = df.n_gblocks;
         df.part_off = pl.fwd_part_floats;
@@ -297,7 +324,7 @@ void fill_batches(Plan& pl, const fmb_params* p, const long long* offs, int n_vi
       bf.v[i] = df;
       // backward
       fmb::DevView db = d;
-      BwdBlocking bk = bwd_blocking(d.K, pl.bwd_threads, p->bwd_gblocks, p->store_pairs != 0);
+      BwdBlocking bk = bwd_blocking(d.K, pl.bwd_threads, p->bwd_gblocks, even_blocks(p, pl));
       if (ac) bk = BwdBlocking{1, d.K, 1};  // one 32-ray tile x all K Gaussians per item
       const int tile_b = ac ? fmb::ac_rays_per_item() : pl.ray_tile;
       db.n_tiles = static_cast<int>((P + tile_b - 1) / tile_b);
@@ -344,7 +371,10 @@ Plan make_plan(const fmb_params* p, const long long* offs, int n_objects, int n_
                bool allow_big = false) {
   Plan pl;
   pl.rpt = p->fwd_rays_per_thread > 0 ? p->fwd_rays_per_thread : kDefaultRpt;
-  pl.bwd_threads = p->bwd_threads > 0 ? p->bwd_threads : choose_bwd_threads(views, n_views, offs, p->bwd_gblocks, p->store_pairs != 0);
+  pl.world = p->variant == 0 && (p->store_pairs || total_entries(views, n_views) <= kWorldRays);
+  pl.bwd_threads = p->bwd_threads > 0
+                       ? p->bwd_threads
+                       : choose_bwd_threads(views, n_views, offs, p->bwd_gblocks, even_blocks(p, pl));
   // default ray tile: three rays per thread in the per-ray phase (balanced, and long
   // enough to amortise the per-CTA reductions)
   pl.ray_tile = p->bwd_ray_tile > 0 ? p->bwd_ray_tile : 3 * pl.bwd_threads;
@@ -442,6 +472,18 @@ fmb::Consts make_consts(const fmb_params* p) {
   c.beta1 = p->beta1;
   c.b2e = static_cast<float>(static_cast<double>(p->beta2) / p->eta);
   return c;
+}
+
+// The prologue of a render or adjoint call: the records its kernels read
+// (camera-plane or world-frame ones).
+template <class B>
+cudaError_t launch_records(const fmb_params* p, const Plan& pl, const B& b, const fmb::Scene& sc, const fmb::Consts& c,
+                           float4* records, int* status_to_clear, int* counter, cudaStream_t s,
+                           const fmb::ZeroJob* zero) {
+  const int maxK = pl.maxK;
+  if (p->variant == 1 || pl.world)
+    return fmb::launch_prologue(b, sc, c, records, maxK, status_to_clear, counter, s, zero);
+  return fmb::launch_prologue_cam(b, sc, records, maxK, status_to_clear, counter, s, zero);
 }
 
 fmb_status check_workspace(void* ws, size_t bytes, size_t need) {
@@ -565,7 +607,7 @@ fmb_status fmb_render_forward(const fmb_params* params, int n_objects, const lon
     auto run = [&](const auto& fwd, const auto& fmerge) -> fmb_status {
       for (size_t bi = 0; bi < fwd.size(); ++bi) {
         const auto& b = fwd[bi];
-        e = fmb::launch_prologue(b, sc, c, records, pl.maxK, bi == 0 ? status : nullptr, counter, s);
+        e = launch_records(params, pl, b, sc, c, records, bi == 0 ? status : nullptr, counter, s, nullptr);
         if (e != cudaSuccess) return cuda_fail(e, "prologue launch");
         fmb::FwdOut fo{depth, alpha, normal, flow, saved, pairs, pl.pair_stride};
         fo.color = color;
@@ -580,10 +622,14 @@ fmb_status fmb_render_forward(const fmb_params* params, int n_objects, const lon
             continue;
           }
         }
-        e = fmb::launch_forward(b, sc, c, records, params->want_normals != 0, params->n_flow, pl.rpt, pl.maxK, fo,
-                                status, counter, s);
+        const bool normals = params->want_normals != 0;
+        e = pl.world ? fmb::launch_forward_world(b, sc, c, records, normals, params->n_flow, pl.rpt, pl.maxK, fo, status,
+                                                 counter, s)
+                     : fmb::launch_forward(b, sc, c, records, normals, params->n_flow, pl.rpt, pl.maxK, fo, status,
+                                           counter, s);
         if (e == cudaSuccess && pl.ksplit > 1)
-          e = fmb::launch_forward_merge(fmerge[bi], sc, params->want_normals != 0, params->n_flow, fo, s);
+          e = pl.world ? fmb::launch_forward_merge_world(fmerge[bi], sc, normals, params->n_flow, fo, s)
+                       : fmb::launch_forward_merge(fmerge[bi], sc, c, normals, params->n_flow, fo, s);
         if (e != cudaSuccess) return cuda_fail(e, "forward launch");
       }
       return FMB_OK;
@@ -667,7 +713,7 @@ fmb_status fmb_render_backward(const fmb_params* params, int n_objects, const lo
     // batches: pl.bwd, or its 256-view counterpart
     auto run = [&](const auto& bwd) -> fmb_status {
       for (const auto& b : bwd) {
-        e = fmb::launch_prologue(b, sc, c, records, pl.maxK, nullptr, counter, s, first ? &zj : nullptr);
+        e = launch_records(params, pl, b, sc, c, records, nullptr, counter, s, first ? &zj : nullptr);
         first = false;
         if (e != cudaSuccess) return cuda_fail(e, "prologue launch");
         bool done = false;
@@ -679,8 +725,10 @@ fmb_status fmb_render_backward(const fmb_params* params, int n_objects, const lo
           }
         }
         if (!done)
-          e = fmb::launch_backward(b, sc, c, records, normals, params->n_flow, pl.ray_tile, pl.bwd_threads, in, out,
-                                   counter, s);
+          e = pl.world ? fmb::launch_backward_world(b, sc, c, records, normals, params->n_flow, pl.ray_tile,
+                                                    pl.bwd_threads, in, out, counter, s)
+                       : fmb::launch_backward(b, sc, c, records, normals, params->n_flow, pl.ray_tile, pl.bwd_threads, in,
+                                              out, counter, s);
         if (e != cudaSuccess) return cuda_fail(e, "backward launch");
         if (partials) {
           e = fmb::launch_backward_reduce(b, params->n_flow, pl.n_gauss, n_poses, out, s);
@@ -860,7 +908,10 @@ fmb_status fmb_read_device_status(const void* workspace, int* h_status, fmb_stre
 
 namespace {
 
-constexpr size_t kStaticScratchBytes = size_t(1) << 20;  // 1 MiB
+// The limit on a batch is 1 MiB by its Gaussians (64 bytes per view and Gaussian); the
+// array also holds one padding record per view of an odd count, at most as many again.
+constexpr size_t kStaticScratchLimit = size_t(1) << 20;
+constexpr size_t kStaticScratchBytes = 2 * kStaticScratchLimit;
 constexpr int kStaticMaxDevices = 64;
 
 static __device__ __align__(256) unsigned char g_fmb_static_scratch[kStaticScratchBytes];
@@ -913,10 +964,11 @@ extern "C" fmb_status fmb_render_forward_noalloc(const fmb_params* params, int n
     Plan pl = make_plan(params, h_obj_offsets, n_objects, n_views, h_views);
     if (params->colors && (!colors || !color))
       return fail(FMB_ERR_INVALID_ARG, "colors and color are required when params->colors is set");
-    const size_t need = partials_offset(params, pl);
-    if (need > kStaticScratchBytes)
+    size_t need = kHeaderBytes + align256(static_cast<size_t>(pl.n_pairs) * 16 * fmb::kRecFloat4);
+    if (params->colors) need += align256(static_cast<size_t>(pl.n_pairs) * 16);
+    if (need > kStaticScratchLimit || partials_offset(params, pl) > kStaticScratchBytes)
       return fail(FMB_ERR_WORKSPACE, "batch needs " + std::to_string(need) + " bytes of scratch; the static scratch " +
-                                         "holds " + std::to_string(kStaticScratchBytes) +
+                                         "holds " + std::to_string(kStaticScratchLimit) +
                                          " (64 bytes per view and Gaussian, 80 with colours, plus 256)");
     void* ws = nullptr;
     st = static_scratch_address(&ws);
@@ -939,7 +991,7 @@ extern "C" fmb_status fmb_render_forward_noalloc(const fmb_params* params, int n
                        : nullptr;
     for (size_t bi = 0; bi < pl.fwd.size(); ++bi) {
       const fmb::Batch& b = pl.fwd[bi];
-      e = fmb::launch_prologue(b, sc, c, records, pl.maxK, bi == 0 ? status : nullptr, counter, s);
+      e = launch_records(params, pl, b, sc, c, records, bi == 0 ? status : nullptr, counter, s, nullptr);
       if (e != cudaSuccess) return cuda_fail(e, "prologue launch");
       fmb::FwdOut fo{depth, alpha, normal, flow, saved, pairs, pl.pair_stride};
       fo.color = color;
@@ -948,8 +1000,10 @@ extern "C" fmb_status fmb_render_forward_noalloc(const fmb_params* params, int n
         e = fmb::launch_forward_ac(b, sc, c, records, params->want_normals != 0, params->n_flow, pl.maxK, fo, pl.ac_run,
                                    status, counter, s);
       } else {
-        e = fmb::launch_forward(b, sc, c, records, params->want_normals != 0, params->n_flow, pl.rpt, pl.maxK, fo,
-                                status, counter, s);
+        e = pl.world ? fmb::launch_forward_world(b, sc, c, records, params->want_normals != 0, params->n_flow, pl.rpt,
+                                                 pl.maxK, fo, status, counter, s)
+                     : fmb::launch_forward(b, sc, c, records, params->want_normals != 0, params->n_flow, pl.rpt, pl.maxK,
+                                           fo, status, counter, s);
       }
       if (e != cudaSuccess) return cuda_fail(e, "forward launch");
     }

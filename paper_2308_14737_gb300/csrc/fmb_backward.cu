@@ -17,19 +17,27 @@
 // into gradients of mu, L, lambda and of the pose, and writes them once per CTA
 // (fp32 atomics, or per-CTA partials that a second kernel adds in a fixed order).
 //
-// Adjoint in the whitened form (a = L^T v, b = L^T (mu - o), t = a.b/a.a,
-// u = t a - b, q = u.u, g = L u, n = g/|g|, what = softmax of e):
+// Adjoint in the camera-plane form of fmb_cam.cuh (a = B^T c, D = B^T d3 with
+// d3 = z c - m, t = z + tau, u = D + tau a, g = B u, n = g/|g|, what = softmax of e):
 //   ebar  = what (Dbar (t - D) + Nbar . n)            (softmax of Eq. 3)
 //   dbar  = beta1 ebar + Abar e^{-sum delta} delta     (Eq. 7, Eq. 8)
-//   tbar  = Dbar what - (beta2/eta) ebar + (L^T gbar) . a
 //   gbar  = what/|g| (Nbar - (n . Nbar) n)             (Eq. 17 normalisation)
-//   ubar  = L^T gbar - dbar u
-//   y     = ubar - (tbar/a.a) a,  bbar = -y,  abar = t y - (tbar/a.a) u
-// and per Gaussian: Lbar = lower(sum gbar u^T + sum v abar^T + (mu - o) bbar^T),
-// mubar = L sum bbar, lambdabar = sum dbar / lambda.  The term -dbar u . a of tbar
-// is dropped: u . a = 0 exactly at the max-likelihood depth.
+//   tbar  = Dbar what - (beta2/eta) ebar + (B^T gbar) . a
+//   ubar  = B^T gbar - dbar u,   s = -tbar / a.a
+//   y     = Dbar_vec = ubar + s a,   abar = tau y + s u
+// (the contribution -dbar u.a of tbar is dropped: u . a = 0 exactly at the
+// max-likelihood depth).  Since n is perpendicular to c and B is triangular, gbar
+// needs the first two components only, and u's third enters through
+// sigma = s - dbar tau and kappa = tau (sigma + s) alone (abar_2 = kappa e2,
+// y_2 = sigma e2).  The render depends on B only through P = B B^T, so the gradient
+// with respect to a full 3x3 root is X B with X symmetric (X = 2 Pbar), and the six
+// lower entries that are accumulated give X by substitution; then Lbar =
+// lower(R^T X A) and Rbar = X A L^T with A = R L, and the mean's gradient comes from
+// sum y.  Ten sums per Gaussian instead of the nineteen of the world-frame form, and with
+// normals and pose gradients five more (below).
 #include <algorithm>
 
+#include "fmb_cam.cuh"
 #include "fmb_f32x2.cuh"
 #include "fmb_internal.cuh"
 
@@ -44,136 +52,128 @@ constexpr int kBwdMaxThreads = 160;
 #endif
 constexpr int kBwdMinBlocks = FMB_BWD_MIN_BLOCKS;  // resident CTAs per SM the register budget targets
 constexpr int kBwdUnroll = FMB_BWD_UNROLL;
-constexpr int kAccFloats = 38;  // 19 packed accumulators per thread in the reduction
-// Colour mode adds three (sum of what x Cbar per channel).
-template <bool COLOR>
-__host__ __device__ constexpr int acc_floats() {
-  return COLOR ? 44 : kAccFloats;
-}
 
-// Per-thread gradient sums of the thread's two Gaussians (one per lane).
+// Per-thread gradient sums of the thread's two Gaussians (one per lane).  y, abar,
+// B00 .. are scaled and in pixels as the records are (fmb_cam.cuh).
+//   0 A00  1 A10  2 A11   sum dx p0 + gb0 u0, dy p0 + gb1 u0, dy p1 + gb1 u1 (p = t y + s u)
+//   3 Y0   4 Y1   5 Sg    sum y, sum sigma
+//   6 E0   7 E1   8 Kp    sum abar, sum kappa (abar from sum p - z sum y instead costs
+//                         two operations less and three times the error of Lbar)
+//   9 nd                  -2 ln 2 sum dbar
+//   NORMALS with pose gradients: T00 T01 T11 V0 V1, sum over the pairs of
+//     what (n . Nbar) n n^T / |g|^2 in the first two components, and of its products
+//     with dx h0 + dy h1 (for the third)
+//   COLOR: sum what Cbar (3)
+constexpr int kAccBase = 10;
+template <bool NORMALS, bool COLOR, bool POSE>
+__host__ __device__ constexpr int acc_count() {
+  return kAccBase + (NORMALS && POSE ? 5 : 0) + (COLOR ? 3 : 0);
+}
+template <bool NORMALS, bool COLOR, bool POSE>
 struct BwdAcc2 {
-  f2 nSd;                 // -sum dbar
-  f2 Y0, Y1, Y2;          // sum y   (= -sum bbar)
-  f2 G00, G10, G11, G20, G21, G22;  // sum gbar u^T (lower)
-  f2 M[9];                // sum v abar^T (row-major)
-  f2 Cb0, Cb1, Cb2;       // colour mode: sum what Cbar
+  static constexpr int kN = acc_count<NORMALS, COLOR, POSE>();
+  static constexpr int kT = kAccBase, kCol = kN - 3;
+  f2 v[kN];
 };
 
-// Shared-memory record of one ray, 7 x 16 bytes, every value duplicated:
-//   [v0 v0 v1 v1 | v2 v2 -lse2 -lse2 | Dbar Dbar -KA -KA | -C -C Nb0 Nb0 |
-//    Nb1 Nb1 Nb2 Nb2 | vl0 vl0 vl1 vl1 | vl2 vl2 0 0]
-// Colour mode: 8 x 16 bytes, the last two [vl2 vl2 Cb0 Cb0 | Cb1 Cb1 Cb2 Cb2].
-constexpr int kRayRec2 = 7;
-template <bool COLOR>
+// Shared-memory record of one ray, every value duplicated so that one 16-byte load
+// gives two broadcast pairs:
+//   [X Y | -lse2 K2 | Dbar -D | -KA -B2E]
+//   NORMALS: [Nt0 Nt1 | m00 m01 | m11 0]      COLOR: [Cb0 Cb1 | Cb2 -Cbar.C]
+// X, Y: pixel centre.  K2 = -(beta2/eta) log2(e) |c|, B2E = (beta2/eta) |c|, Dbar the
+// depth's upstream gradient times |c| (t is measured along z), D the depth along z
+// (t - D is formed first: it is exact where one Gaussian is seen), KA = 2 ln 2 Abar
+// e^-sum delta.  Nt = (fx (Nbar_0 - x Nbar_2), fy (Nbar_1 - y Nbar_2)): Nbar applied
+// to the image-plane components h of g.  m: minus the quadratic form |g|^2 of h.
+template <bool NORMALS, bool COLOR>
 __host__ __device__ constexpr int ray_rec2() {
-  return COLOR ? 8 : kRayRec2;
+  return 4 + (NORMALS ? 3 : 0) + (COLOR ? 2 : 0);
 }
 
-// STORED: the pair's t, log2 weight and density come from the forward (`st`,
-// `se`, `sd`) instead of being recomputed.  POSE = false (no pose gradient
-// requested): only the lower triangle of sum v abar^T is needed, for Lbar, so it
-// is accumulated together with sum gbar u^T into the six G sums and M stays zero.
-template <bool NORMALS, bool STORED, bool COLOR = false, bool POSE = true>
-__device__ __forceinline__ void bwd_pair2(BwdAcc2& A, const GaussRec2& gr, const ulonglong2* __restrict__ rr, f2 K2,
-                                          f2 K3, f2 B1, f2 nB1, f2 nB2E, f2 tiny, f2 st, f2 se, f2 sd,
-                                          f2 c0 = f2{}, f2 c1 = f2{}, f2 c2 = f2{}) {
-  const ulonglong2 q0 = rr[0], q1 = rr[1], q2 = rr[2], q3 = rr[3], q4 = rr[4], q5 = rr[5], q6 = rr[6];
-  // colour mode: Cbar . c_i joins the weight's gradient (Eq. 3 with colours)
-  f2 cc = dup(0.f), Cb0 = dup(0.f), Cb1 = dup(0.f), Cb2 = dup(0.f);
-  if (COLOR) {
-    const ulonglong2 q7 = rr[7];
-    Cb0 = as_f2(q6.y);
-    Cb1 = as_f2(q7.x);
-    Cb2 = as_f2(q7.y);
-    cc = fma2(Cb2, c2, fma2(Cb1, c1, mul2(Cb0, c0)));
-  }
-  const f2 v0 = as_f2(q0.x), v1 = as_f2(q0.y), v2 = as_f2(q1.x), nlse = as_f2(q1.y);
-  const f2 Dbar = as_f2(q2.x), nKA = as_f2(q2.y), nC = as_f2(q3.x);
-  PairGeom2 G;
-  f2 what, delta;
-  if (STORED) {
-    G = pair_geom2_given_t<NORMALS>(gr, st, v0, v1, v2, as_f2(q5.x), as_f2(q5.y), as_f2(q6.x));
-    what = ex2_2(add2(se, nlse));
-    delta = sd;
-  } else {
-    G = pair_geom2<NORMALS>(gr, v0, v1, v2, as_f2(q5.x), as_f2(q5.y), as_f2(q6.x));
-    const f2 x = fma2(G.q, K3, gr.l2);  // log2(delta)
-    what = ex2_2(fma2(x, B1, fma2(G.t, K2, nlse)));
-    delta = ex2_2(x);
-  }
-  const f2 t = G.t;
-  f2 ebar, ub0, ub1, ub2, tbar, gb0, gb1, gb2;
+template <bool NORMALS, bool COLOR, bool POSE>
+__device__ __forceinline__ void bwd_pair2(BwdAcc2<NORMALS, COLOR, POSE>& S, const CamRec2& g,
+                                          const ulonglong2* __restrict__ rr, f2 nB1, f2 nB1s, f2 tiny, f2 c0,
+                                          f2 c1, f2 c2) {
+  using Acc = BwdAcc2<NORMALS, COLOR, POSE>;
+  const ulonglong2 q0 = rr[0], q1 = rr[1], q2 = rr[2], q3 = rr[3];
+  const f2 nlse = as_f2(q1.x), K2 = as_f2(q1.y), Dbar = as_f2(q2.x), nD = as_f2(q2.y), nKA = as_f2(q3.x),
+           nB2E = as_f2(q3.y);
+  const CamGeom2 G = cam_geom2(g, as_f2(q0.x), as_f2(q0.y));
+  const f2 what = ex2_2(fma2(G.t, K2, fma2(G.nx, nB1, nlse)));
+  const f2 delta = pk(ex2_approx(-lo(G.nx)), ex2_approx(-hi(G.nx)));
+  const f2 Dw = mul2(Dbar, what), tD = add2(G.t, nD);
+  f2 br;  // the bracket of ebar, unless it is the depth's term alone
+  f2 rs, nN, h0, h1, m0, m1, Nt0, Nt1;
   if (NORMALS) {
-    const f2 Nb0 = as_f2(q3.y), Nb1 = as_f2(q4.x), Nb2 = as_f2(q4.y);
-    const f2 g0 = mul2(gr.L[0], G.u0);
-    const f2 g1 = fma2(gr.L[2], G.u1, mul2(gr.L[1], G.u0));
-    const f2 g2 = fma2(gr.L[5], G.u2, fma2(gr.L[4], G.u1, mul2(gr.L[3], G.u0)));
-    const f2 gg = add2(fma2(g2, g2, fma2(g1, g1, mul2(g0, g0))), tiny);
-    const f2 rs = rsqrt_2(gg);
-    const f2 n0 = mul2(g0, rs), n1 = mul2(g1, rs), n2 = mul2(g2, rs);
-    const f2 nN = fma2(n2, Nb2, fma2(n1, Nb1, mul2(n0, Nb0)));
-    ebar = mul2(what, COLOR ? add2(add2(fma2(Dbar, t, nC), nN), cc) : add2(fma2(Dbar, t, nC), nN));
+    const ulonglong2 q4 = rr[4], q5 = rr[5], q6 = rr[6];
+    Nt0 = as_f2(q4.x);
+    Nt1 = as_f2(q4.y);
+    h0 = mul2(g.B00, G.u0);
+    h1 = fma2(g.B11, G.u1, mul2(g.B10, G.u0));
+    m0 = fma2(as_f2(q5.y), h1, mul2(as_f2(q5.x), h0));  // minus the metric times h
+    m1 = fma2(as_f2(q6.x), h1, mul2(as_f2(q5.y), h0));
+    const f2 ngg = fma2(h0, m0, fma2(h1, m1, tiny));    // -|g|^2 (tiny < 0)
+    rs = pk(rsqrt_approx(-lo(ngg)), rsqrt_approx(-hi(ngg)));
+    nN = mul2(fma2(Nt0, h0, mul2(Nt1, h1)), rs);
+    br = fma2(Dbar, tD, nN);
+  }
+  f2 Cb0, Cb1, Cb2;
+  if (COLOR) {  // Cbar . c_i joins the weight's gradient (Eq. 3 with colours)
+    const ulonglong2 q7 = rr[NORMALS ? 7 : 4], q8 = rr[NORMALS ? 8 : 5];
+    Cb0 = as_f2(q7.x);
+    Cb1 = as_f2(q7.y);
+    Cb2 = as_f2(q8.x);
+    const f2 cc = fma2(Cb2, c2, fma2(Cb1, c1, fma2(Cb0, c0, as_f2(q8.y))));
+    br = NORMALS ? add2(br, cc) : fma2(Dbar, tD, cc);
+  }
+  const f2 ebar = NORMALS || COLOR ? mul2(what, br) : mul2(Dw, tD);
+  const f2 nd = fma2(nB1s, ebar, mul2(nKA, delta));
+  f2 tbar = fma2(nB2E, ebar, Dw);
+  f2 ub0, ub1;
+  if (!NORMALS) {
+    ub0 = mul2(nd, G.u0);
+    ub1 = mul2(nd, G.u1);
+  } else {
     const f2 sc = mul2(what, rs);
-    const f2 sN = mul2(sc, nN);
-    const f2 nsN = pk(-lo(sN), -hi(sN));
-    gb0 = fma2(nsN, n0, mul2(sc, Nb0));
-    gb1 = fma2(nsN, n1, mul2(sc, Nb1));
-    gb2 = fma2(nsN, n2, mul2(sc, Nb2));
-    ub0 = fma2(gr.L[3], gb2, fma2(gr.L[1], gb1, mul2(gr.L[0], gb0)));
-    ub1 = fma2(gr.L[4], gb2, mul2(gr.L[2], gb1));
-    ub2 = mul2(gr.L[5], gb2);
-    tbar = fma2(ub2, G.a2, fma2(ub1, G.a1, fma2(ub0, G.a0, fma2(Dbar, what, mul2(nB2E, ebar)))));
-  } else {
-    ebar = mul2(what, COLOR ? add2(fma2(Dbar, t, nC), cc) : fma2(Dbar, t, nC));
-    ub0 = ub1 = ub2 = gb0 = gb1 = gb2 = dup(0.f);
-    tbar = fma2(Dbar, what, mul2(nB2E, ebar));
-  }
-  const f2 ndbar = fma2(nB1, ebar, mul2(nKA, delta));  // -dbar
-  ub0 = fma2(ndbar, G.u0, ub0);
-  ub1 = fma2(ndbar, G.u1, ub1);
-  ub2 = fma2(ndbar, G.u2, ub2);
-  const f2 ns2 = mul2(tbar, G.ninv);  // -tbar / a.a
-  const f2 y0 = fma2(ns2, G.a0, ub0);
-  const f2 y1 = fma2(ns2, G.a1, ub1);
-  const f2 y2 = fma2(ns2, G.a2, ub2);
-  const f2 ab0 = fma2(t, y0, mul2(ns2, G.u0));
-  const f2 ab1 = fma2(t, y1, mul2(ns2, G.u1));
-  const f2 ab2 = fma2(t, y2, mul2(ns2, G.u2));
-  A.nSd = add2(A.nSd, ndbar);
-  A.Y0 = add2(A.Y0, y0);
-  A.Y1 = add2(A.Y1, y1);
-  A.Y2 = add2(A.Y2, y2);
-  if (POSE) {
-    if (NORMALS) {
-      A.G00 = fma2(gb0, G.u0, A.G00);
-      A.G10 = fma2(gb1, G.u0, A.G10);
-      A.G11 = fma2(gb1, G.u1, A.G11);
-      A.G20 = fma2(gb2, G.u0, A.G20);
-      A.G21 = fma2(gb2, G.u1, A.G21);
-      A.G22 = fma2(gb2, G.u2, A.G22);
+    const f2 sN = mul2(mul2(sc, rs), nN);
+    const f2 gb0 = fma2(sN, m0, mul2(sc, Nt0));
+    const f2 gb1 = fma2(sN, m1, mul2(sc, Nt1));
+    const f2 b0 = fma2(g.B10, gb1, mul2(g.B00, gb0));
+    const f2 b1 = mul2(g.B11, gb1);
+    tbar = fma2(b1, G.a1, fma2(b0, G.a0, tbar));
+    ub0 = fma2(nd, G.u0, b0);
+    ub1 = fma2(nd, G.u1, b1);
+    S.v[0] = fma2(gb0, G.u0, S.v[0]);
+    S.v[1] = fma2(gb1, G.u0, S.v[1]);
+    S.v[2] = fma2(gb1, G.u1, S.v[2]);
+    if (POSE) {
+      const f2 r0 = mul2(sN, h0), r1 = mul2(sN, h1), w = fma2(G.dx, h0, mul2(G.dy, h1));
+      S.v[Acc::kT + 0] = fma2(r0, h0, S.v[Acc::kT + 0]);
+      S.v[Acc::kT + 1] = fma2(r0, h1, S.v[Acc::kT + 1]);
+      S.v[Acc::kT + 2] = fma2(r1, h1, S.v[Acc::kT + 2]);
+      S.v[Acc::kT + 3] = fma2(r0, w, S.v[Acc::kT + 3]);
+      S.v[Acc::kT + 4] = fma2(r1, w, S.v[Acc::kT + 4]);
     }
-    A.M[0] = fma2(v0, ab0, A.M[0]);
-    A.M[1] = fma2(v0, ab1, A.M[1]);
-    A.M[2] = fma2(v0, ab2, A.M[2]);
-    A.M[3] = fma2(v1, ab0, A.M[3]);
-    A.M[4] = fma2(v1, ab1, A.M[4]);
-    A.M[5] = fma2(v1, ab2, A.M[5]);
-    A.M[6] = fma2(v2, ab0, A.M[6]);
-    A.M[7] = fma2(v2, ab1, A.M[7]);
-    A.M[8] = fma2(v2, ab2, A.M[8]);
-  } else {
-    A.G00 = fma2(v0, ab0, NORMALS ? fma2(gb0, G.u0, A.G00) : A.G00);
-    A.G10 = fma2(v1, ab0, NORMALS ? fma2(gb1, G.u0, A.G10) : A.G10);
-    A.G11 = fma2(v1, ab1, NORMALS ? fma2(gb1, G.u1, A.G11) : A.G11);
-    A.G20 = fma2(v2, ab0, NORMALS ? fma2(gb2, G.u0, A.G20) : A.G20);
-    A.G21 = fma2(v2, ab1, NORMALS ? fma2(gb2, G.u1, A.G21) : A.G21);
-    A.G22 = fma2(v2, ab2, NORMALS ? fma2(gb2, G.u2, A.G22) : A.G22);
   }
+  const f2 s = mul2(tbar, G.ninv);  // -tbar / a.a
+  const f2 y0 = fma2(s, G.a0, ub0), y1 = fma2(s, G.a1, ub1);
+  const f2 su0 = mul2(s, G.u0), su1 = mul2(s, G.u1);
+  const f2 p0 = fma2(G.t, y0, su0), p1 = fma2(G.t, y1, su1);  // z y + abar
+  const f2 sg = fma2(nd, G.tau, s);
+  S.v[0] = fma2(G.dx, p0, S.v[0]);
+  S.v[1] = fma2(G.dy, p0, S.v[1]);
+  S.v[2] = fma2(G.dy, p1, S.v[2]);
+  S.v[3] = add2(S.v[3], y0);
+  S.v[4] = add2(S.v[4], y1);
+  S.v[5] = add2(S.v[5], sg);
+  S.v[6] = add2(S.v[6], fma2(G.tau, y0, su0));
+  S.v[7] = add2(S.v[7], fma2(G.tau, y1, su1));
+  S.v[8] = fma2(G.tau, add2(sg, s), S.v[8]);
+  S.v[9] = add2(S.v[9], nd);
   if (COLOR) {
-    A.Cb0 = fma2(what, Cb0, A.Cb0);
-    A.Cb1 = fma2(what, Cb1, A.Cb1);
-    A.Cb2 = fma2(what, Cb2, A.Cb2);
+    S.v[Acc::kCol + 0] = fma2(what, Cb0, S.v[Acc::kCol + 0]);
+    S.v[Acc::kCol + 1] = fma2(what, Cb1, S.v[Acc::kCol + 1]);
+    S.v[Acc::kCol + 2] = fma2(what, Cb2, S.v[Acc::kCol + 2]);
   }
 }
 
@@ -183,9 +183,109 @@ __device__ __forceinline__ float warp_sum(float x) {
   return x;
 }
 
+// A Gaussian's gradients from its summed accumulators: X of the header from the lower
+// entries of X B' in the offsets' frame, brought to the camera frame (c = S c', S =
+// [[1/fx, 0, xe], [0, 1/fy, ye], [0, 0, 1]]), then Lbar = lower(R^T X A), mubar = R^-1
+// mbar, and the pose: Rbar = X A L^T - (R^-T mu) mubar^T (+ the normal's term), tbar =
+// mbar, as functions of a general R (A = R L, m = R^-T mu + t).
+template <bool NORMALS, bool COLOR, bool POSE>
+__device__ __forceinline__ void bwd_finalise(const Scene& s, const DevView& V, const float4* __restrict__ records,
+                                             const float* view_inv, int g, const float* acc, bool want_pose, float gm[3],
+                                             float gL[6], float& glam, float pose_g[12]) {
+  using Acc = BwdAcc2<NORMALS, COLOR, POSE>;
+  const long long gg = V.gauss_off + g;
+  const float* rec = reinterpret_cast<const float*>(records) +
+                     2 * kCamF2 * ((static_cast<long long>(V.rec_off) + g) >> 1) + (g & 1);
+  const float pex = -rec[0], pey = -rec[2], B00 = rec[4], B10 = rec[6], e0 = rec[12], B11 = rec[14],
+              e1 = rec[16], ee = rec[22], rho0 = rec[28], rho1 = rec[30];
+  const float Y0 = acc[3], Y1 = acc[4], Kp = acc[8];
+  // lower entries of X B' in the offsets' frame
+  const float b00 = fmaf(-rho0, Y0, acc[0]), b10 = fmaf(-rho1, Y0, acc[1]), b11 = fmaf(-rho1, Y1, acc[2]);
+  const float b20 = acc[6], b21 = acc[7];
+  const float i0 = B00 != 0.f ? 1.0f / B00 : 0.f, i1 = B11 != 0.f ? 1.0f / B11 : 0.f;
+  const float X22 = Kp;
+  const float X21 = fmaf(-X22, e1, b21) * i1;
+  const float X11 = fmaf(-X21, e1, b11) * i1;
+  const float X20 = fmaf(-X22, e0, fmaf(-X21, B10, b20)) * i0;
+  const float X10 = fmaf(-X21, e0, fmaf(-X11, B10, b10)) * i0;
+  const float X00 = fmaf(-X20, e0, fmaf(-X10, B10, b00)) * i0;
+  // camera frame: S X S^T, with the scale of the whitened quantities
+  const float ifx = 1.0f / V.fx, ify = 1.0f / V.fy, px = pex - V.cx, py = pey - V.cy;
+  const float xe = px * ifx, ye = py * ify;
+  const float t0 = X20 * ifx, t1 = X21 * ify;
+  float X[9];
+  X[8] = kCamScale2 * X22;
+  X[6] = kCamScale2 * fmaf(xe, X22, t0);
+  X[7] = kCamScale2 * fmaf(ye, X22, t1);
+  X[0] = fmaf(kCamScale2, fmaf(X00 * ifx, ifx, xe * t0), xe * X[6]);
+  X[4] = fmaf(kCamScale2, fmaf(X11 * ify, ify, ye * t1), ye * X[7]);
+  X[1] = fmaf(kCamScale2, fmaf(X10 * ifx, ify, xe * t1), ye * X[6]);
+  X[2] = X[6];
+  X[3] = X[1];
+  X[5] = X[7];
+  float R[9], tp[3];
+  load_pose(s.poses, V.pose, R, tp);
+  const float* Lp = s.chol + 6 * gg;
+  const float L00 = Lp[0], L10 = Lp[1], L11 = Lp[2], L20 = Lp[3], L21 = Lp[4], L22 = Lp[5];
+  float XA[9];  // X A = Abar
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    float XR[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) XR[c] = fmaf(X[3 * a + 2], R[6 + c], fmaf(X[3 * a + 1], R[3 + c], X[3 * a] * R[c]));
+    XA[3 * a + 0] = fmaf(XR[2], L20, fmaf(XR[1], L10, XR[0] * L00));
+    XA[3 * a + 1] = fmaf(XR[2], L21, XR[1] * L11);
+    XA[3 * a + 2] = XR[2] * L22;
+  }
+  auto RtXA = [&](int a, int c) { return fmaf(R[6 + a], XA[6 + c], fmaf(R[3 + a], XA[3 + c], R[a] * XA[c])); };
+  gL[0] = RtXA(0, 0);
+  gL[1] = RtXA(1, 0);
+  gL[2] = RtXA(1, 1);
+  gL[3] = RtXA(2, 0);
+  gL[4] = RtXA(2, 1);
+  gL[5] = RtXA(2, 2);
+  glam = -acc[9] / (kTwoLn2 * s.weights[gg]);
+  // mbar = -B sum y; B's last row from e0, e1
+  const float B20 = fmaf(-B10, py, fmaf(-B00, px, e0)), B21 = fmaf(-B11, py, e1);
+  float mb[3];
+  mb[0] = -V.fx * B00 * Y0;
+  mb[1] = -V.fy * fmaf(B11, Y1, B10 * Y0);
+  mb[2] = -fmaf(ee, acc[5], fmaf(B21, Y1, B20 * Y0));
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    gm[c] = fmaf(view_inv[3 * c + 2], mb[2], fmaf(view_inv[3 * c + 1], mb[1], view_inv[3 * c] * mb[0]));
+  if (!POSE || !want_pose) return;
+  const float mu0 = s.means[3 * gg], mu1 = s.means[3 * gg + 1], mu2 = s.means[3 * gg + 2];
+  float T[9];
+  if (NORMALS) {  // sum what (n . Nbar) n n^T, the third component from n . c = 0, its trace 0
+    const float T00 = acc[Acc::kT], T01 = acc[Acc::kT + 1], T11 = acc[Acc::kT + 2];
+    const float V0 = fmaf(px, T00, fmaf(py, T01, acc[Acc::kT + 3])), V1 = fmaf(px, T01, fmaf(py, T11, acc[Acc::kT + 4]));
+    T[0] = V.fx * V.fx * T00;
+    T[4] = V.fy * V.fy * T11;
+    T[1] = T[3] = V.fx * V.fy * T01;
+    T[2] = T[6] = -V.fx * V0;
+    T[5] = T[7] = -V.fy * V1;
+    T[8] = -(T[0] + T[4]);
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    // row a of R^-T mu
+    const float rm = fmaf(view_inv[6 + a], mu2, fmaf(view_inv[3 + a], mu1, view_inv[a] * mu0));
+    float row[3] = {XA[3 * a] * L00, fmaf(XA[3 * a + 1], L11, XA[3 * a] * L10),
+                    fmaf(XA[3 * a + 2], L22, fmaf(XA[3 * a + 1], L21, XA[3 * a] * L20))};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      float x = fmaf(-rm, gm[c], row[c]);
+      if (NORMALS) x += fmaf(T[3 * a + 2], R[6 + c], fmaf(T[3 * a + 1], R[3 + c], T[3 * a] * R[c]));
+      pose_g[3 * a + c] += x;
+    }
+    pose_g[9 + a] += mb[a];
+  }
+}
+
 // CL = 2: launched as clusters of two CTAs, the two Gaussian blocks of one ray tile
 // (grid mode, every view of the batch in two blocks); CL = 1: no cluster.
-template <bool NORMALS, int NFLOW, bool STORED, bool COLOR = false, bool POSE = true, int CL = 1, class B = Batch>
+template <bool NORMALS, int NFLOW, bool COLOR = false, bool POSE = true, int CL = 1, class B = Batch>
 __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
     backward_kernel(const __grid_constant__ B batch, Scene s, Consts k, const float4* __restrict__ records,
                     BwdIn in, BwdOut out, int ray_tile, int* counter) {
@@ -194,6 +294,7 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
   constexpr int NPV = 12 * (1 + NFLOW);  // pose values reduced per CTA
   __shared__ float pose_ray[kBwdMaxThreads / 32][NPV];  // per-warp sums of the per-ray pose terms
   __shared__ float pose_gau[kBwdMaxThreads / 32][12];   // per-warp sums of the per-Gaussian pose terms
+  __shared__ float view_inv[9];                         // R^-1 of the view's pose
   __shared__ int s_item;
 
   for (int round = 0;; ++round) {
@@ -230,6 +331,14 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
     const float o0 = -fmaf(R[6], tp[2], fmaf(R[3], tp[1], R[0] * tp[0]));
     const float o1 = -fmaf(R[7], tp[2], fmaf(R[4], tp[1], R[1] * tp[0]));
     const float o2 = -fmaf(R[8], tp[2], fmaf(R[5], tp[1], R[2] * tp[0]));
+    if (tid < 9) {  // entry (a, b) of R^-1 = cof(R)^T / det(R)
+      const int a = tid / 3, b = tid % 3;
+      auto at = [&](int i, int j) { return __ldg(s.poses + 12 * static_cast<long long>(V.pose) + 3 * (i % 3) + j % 3); };
+      const float cof = fmaf(at(b + 1, a + 1), at(b + 2, a + 2), -(at(b + 1, a + 2) * at(b + 2, a + 1)));
+      const float det = fmaf(R[0], fmaf(R[4], R[8], -(R[5] * R[7])),
+                             fmaf(R[1], fmaf(R[5], R[6], -(R[3] * R[8])), R[2] * fmaf(R[3], R[7], -(R[4] * R[6]))));
+      view_inv[tid] = cof / det;
+    }
     float pose_acc[NPV];
 #pragma unroll
     for (int i = 0; i < NPV; ++i) pose_acc[i] = 0.f;
@@ -243,8 +352,12 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
     }
     for (int r = r_lo + tid; r < r_hi; r += T) {
       const int p = pix0 + r;
-      float vc[3], v[3], vl[3], pxy[2];
-      pixel_ray_dd(V, R, ray_pixel(V, p), vc, v, vl, pxy);
+      const CamRay ray = cam_ray(V, ray_pixel(V, p));
+      const float il = 1.0f / ray.len;
+      const float vc[3] = {ray.x * il, ray.y * il, il};
+      float v[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) v[c] = fmaf(R[6 + c], vc[2], fmaf(R[3 + c], vc[1], R[c] * vc[0]));
       const float D = in.depth[off + p];
       const float* sv = in.saved + 3 * off;
       const float lse2 = sv[p];
@@ -301,48 +414,63 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
         const float nc[3] = {nr3[p], nr3[P + p], nr3[2 * P + p]};
         const float gn[3] = {gn3[p], gn3[P + p], gn3[2 * P + p]};
         const float Nn = sv[2 * P + p];
-        // world-frame blended normal and its upstream gradient (R^T applied)
-        float nf[3], nfb[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          nf[c] = fmaf(R[6 + c], nc[2], fmaf(R[3 + c], nc[1], R[c] * nc[0]));
-          nfb[c] = fmaf(R[6 + c], gn[2], fmaf(R[3 + c], gn[1], R[c] * gn[0]));
-        }
+        // Camera frame throughout: Nbar = (gn - (gn . n) n) / |N|.  The rendered normal is
+        // R n_f with n_f formed in the world frame, so a change of R that is not a
+        // rotation also acts through R^-1 g: with the pair terms of phase 2 that adds
+        // [(gn . n) n n^T + sum what (n_i . Nbar) n_i n_i^T] R to the pose's gradient.
+        const float sdot = fmaf(nc[2], gn[2], fmaf(nc[1], gn[1], nc[0] * gn[0]));
         if (ray_pose) {
+          float nR[3];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) nR[c] = sdot * fmaf(R[6 + c], nc[2], fmaf(R[3 + c], nc[1], R[c] * nc[0]));
 #pragma unroll
           for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) pose_acc[3 * a + c] = fmaf(gn[a], nf[c], pose_acc[3 * a + c]);
+            for (int c = 0; c < 3; ++c) pose_acc[3 * a + c] = fmaf(nc[a], nR[c], pose_acc[3 * a + c]);
         }
         if (Nn > 0.f) {
           const float iN = 1.0f / Nn;
-          const float sdot = fmaf(nf[2], nfb[2], fmaf(nf[1], nfb[1], nf[0] * nfb[0]));
-          Nb0 = fmaf(-sdot, nf[0], nfb[0]) * iN;
-          Nb1 = fmaf(-sdot, nf[1], nfb[1]) * iN;
-          Nb2 = fmaf(-sdot, nf[2], nfb[2]) * iN;
+          Nb0 = fmaf(-sdot, nc[0], gn[0]) * iN;
+          Nb1 = fmaf(-sdot, nc[1], gn[1]) * iN;
+          Nb2 = fmaf(-sdot, nc[2], gn[2]) * iN;
         }
       }
-      // Nbar is orthogonal to N, so the softmax centring term is Dbar * D alone (plus
-      // Cbar . C, the blended colour's, in colour mode).
-      float C = Dbar * D;
-      float Cb[3] = {0.f, 0.f, 0.f};
+      // Nbar is orthogonal to N, so the softmax centring terms are Dbar D and, in colour
+      // mode, Cbar . C (the blended colour's).
+      float Cb[3] = {0.f, 0.f, 0.f}, CC = 0.f;
       if (COLOR && in.g_color != nullptr) {
         const float* gc3 = in.g_color + 3 * off;
         const float* cp3 = in.color + 3 * off;
 #pragma unroll
         for (int k3 = 0; k3 < 3; ++k3) {
           Cb[k3] = gc3[k3 * P + p];
-          C = fmaf(Cb[k3], cp3[k3 * P + p], C);
+          CC = fmaf(Cb[k3], cp3[k3 * P + p], CC);
         }
       }
-      const float KA = gA * expf(-Sd);
-      float4* rr = bsm + ray_rec2<COLOR>() * r;
-      const float4 rec[8] = {make_float4(v[0], v[0], v[1], v[1]),     make_float4(v[2], v[2], -lse2, -lse2),
-                             make_float4(Dbar, Dbar, -KA, -KA),       make_float4(-C, -C, Nb0, Nb0),
-                             make_float4(Nb1, Nb1, Nb2, Nb2),         make_float4(vl[0], vl[0], vl[1], vl[1]),
-                             make_float4(vl[2], vl[2], Cb[0], Cb[0]), make_float4(Cb[1], Cb[1], Cb[2], Cb[2])};
+      const float KA = kTwoLn2 * gA * expf(-Sd);
+      const float Dz = Dbar * ray.len, nD = -__fdiv_rn(D, ray.len);
+      constexpr int NR = ray_rec2<NORMALS, COLOR>();
+      const float K2 = __fmul_rn(k.K2, ray.len), b2 = k.b2e * ray.len;
+      float4 rec[NR];
+      rec[0] = make_float4(ray.px, ray.px, ray.py, ray.py);
+      rec[1] = make_float4(-lse2, -lse2, K2, K2);
+      rec[2] = make_float4(Dz, Dz, nD, nD);
+      rec[3] = make_float4(-KA, -KA, -b2, -b2);
+      if constexpr (NORMALS) {
+        const float n0 = V.fx * fmaf(-ray.x, Nb2, Nb0), n1 = V.fy * fmaf(-ray.y, Nb2, Nb1);
+        const float m00 = -V.fx * V.fx * fmaf(ray.x, ray.x, 1.0f), m01 = -V.fx * V.fy * (ray.x * ray.y);
+        const float m11 = -V.fy * V.fy * fmaf(ray.y, ray.y, 1.0f);
+        rec[4] = make_float4(n0, n0, n1, n1);
+        rec[5] = make_float4(m00, m00, m01, m01);
+        rec[6] = make_float4(m11, m11, 0.f, 0.f);
+      }
+      if constexpr (COLOR) {
+        rec[NR - 2] = make_float4(Cb[0], Cb[0], Cb[1], Cb[1]);
+        rec[NR - 1] = make_float4(Cb[2], Cb[2], -CC, -CC);
+      }
+      float4* rr = bsm + NR * r;
 #pragma unroll
-      for (int i = 0; i < ray_rec2<COLOR>(); ++i) {
+      for (int i = 0; i < NR; ++i) {
         rr[i] = rec[i];
         if (CL == 2) st_cluster_f4(rr + i, crank ^ 1, rec[i]);
       }
@@ -367,72 +495,38 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
   const int GB2 = (GB + 1) / 2;  // threads per ray subgroup
   const int gl2 = tid % GB2;
   const int sg = tid / GB2;
-  const int g0 = gb * GB + 2 * gl2;        // lane 0 Gaussian
-  const bool has1 = 2 * gl2 + 1 < GB && g0 + 1 < V.K;  // lane 1 holds a real Gaussian
+  const int g0 = gb * GB + 2 * gl2;  // lane 0 Gaussian (GB is even unless there is one block: whole records)
   const bool active = (sg < S) && (g0 < V.K);
-  BwdAcc2 A;
-  A.nSd = A.Y0 = A.Y1 = A.Y2 = dup(0.f);
-  A.G00 = A.G10 = A.G11 = A.G20 = A.G21 = A.G22 = dup(0.f);
+  using Acc = BwdAcc2<NORMALS, COLOR, POSE>;
+  Acc A;
 #pragma unroll
-  for (int i = 0; i < 9; ++i) A.M[i] = dup(0.f);
-  A.Cb0 = A.Cb1 = A.Cb2 = dup(0.f);
-  GaussRec ga{}, gbr{};
+  for (int i = 0; i < Acc::kN; ++i) A.v[i] = dup(0.f);
   if (active) {
-    const float4* rec = records + kRecFloat4 * (V.rec_off + g0);
-    ga = unpack_rec(rec[0], rec[1], rec[2], rec[3]);
-    if (has1) {
-      const float4* rec1 = rec + kRecFloat4;
-      gbr = unpack_rec(rec1[0], rec1[1], rec1[2], rec1[3]);
-    } else {
-      gbr = ga;  // a copy keeps the unused lane finite; its sums are never written
-    }
-    const GaussRec2 gr = pair_rec(ga, gbr);
-    const f2 K2v = dup(k.K2), K3v = dup(k.K3), B1v = dup(k.beta1), nB1v = dup(-k.beta1), nB2E = dup(-k.b2e);
-    const f2 tiny = dup(1e-30f);
+    const long long rec0 = static_cast<long long>(V.rec_off) + g0;
+    const CamRec2 gr = cam_load(reinterpret_cast<const ulonglong2*>(records + kRecFloat4 * rec0));
+    const f2 nB1 = dup(-k.beta1), nB1s = dup(-kTwoLn2 * k.beta1), tiny = dup(-1e-30f);
     const ulonglong2* rays = reinterpret_cast<const ulonglong2*>(bsm);
-    if (STORED) {
-      // the two Gaussians' stored values are adjacent in the row of pixel p (g0 is even)
-      const unsigned long long* pt =
-          reinterpret_cast<const unsigned long long*>(in.pairs + V.pair_off + static_cast<long long>(pix0) * V.Kp + g0);
-      const long long st2 = in.pair_stride / 2, row2 = V.Kp / 2;
-#pragma unroll kBwdUnroll
-      for (int r = sg; r < nr; r += S) {
-        const unsigned long long* q = pt + static_cast<long long>(r) * row2;
-        bwd_pair2<NORMALS, true>(A, gr, rays + kRayRec2 * r, K2v, K3v, B1v, nB1v, nB2E, tiny, as_f2(__ldg(q)),
-                                 as_f2(__ldg(q + st2)), as_f2(__ldg(q + 2 * st2)));
-      }
-    } else if (COLOR) {
-      // the two Gaussians' colours, one per lane
-      const float4 ca = __ldg(s.crec + V.rec_off + g0), cb = has1 ? __ldg(s.crec + V.rec_off + g0 + 1) : ca;
-      const f2 c0 = pk(ca.x, cb.x), c1 = pk(ca.y, cb.y), c2 = pk(ca.z, cb.z);
-      const f2 z = dup(0.f);
-#pragma unroll kBwdUnroll
-      for (int r = sg; r < nr; r += S)
-        bwd_pair2<NORMALS, false, true>(A, gr, rays + ray_rec2<true>() * r, K2v, K3v, B1v, nB1v, nB2E, tiny, z, z, z,
-                                        c0, c1, c2);
-    } else {
-      const f2 z = dup(0.f);
-#pragma unroll kBwdUnroll
-      for (int r = sg; r < nr; r += S)
-        bwd_pair2<NORMALS, false, false, POSE>(A, gr, rays + kRayRec2 * r, K2v, K3v, B1v, nB1v, nB2E, tiny, z, z, z);
+    constexpr int NR = ray_rec2<NORMALS, COLOR>();
+    f2 c0 = dup(0.f), c1 = c0, c2 = c0;  // the two Gaussians' colours, one per lane
+    if (COLOR) {
+      const ulonglong2* cr = reinterpret_cast<const ulonglong2*>(s.crec + rec0);
+      c0 = as_f2(cr[0].x);
+      c1 = as_f2(cr[0].y);
+      c2 = as_f2(cr[1].x);
     }
+#pragma unroll kBwdUnroll
+    for (int r = sg; r < nr; r += S)
+      bwd_pair2<NORMALS, COLOR, POSE>(A, gr, rays + NR * r, nB1, nB1s, tiny, c0, c1, c2);
   }
   __syncthreads();  // ray records are dead; the shared memory is reused below
 
   // ---------------- phase 3: combine ray subgroups, finalise per Gaussian
-  constexpr int NV = COLOR ? 22 : 19;  // sums per Gaussian
-  constexpr int ACC = acc_floats<COLOR>();
+  constexpr int NV = Acc::kN;          // sums per Gaussian
   constexpr int NC = COLOR ? 13 : 10;  // gradient values per Gaussian in a partial slot
-  float* red = reinterpret_cast<float*>(bsm);
+  f2* red = reinterpret_cast<f2*>(bsm);  // [sum][thread]
   if (sg < S) {
-    float* d = red + ACC * tid;
-    const f2 v[22] = {A.nSd, A.Y0, A.Y1, A.Y2, A.G00, A.G10, A.G11, A.G20, A.G21, A.G22, A.M[0],
-                      A.M[1], A.M[2], A.M[3], A.M[4], A.M[5], A.M[6], A.M[7], A.M[8], A.Cb0, A.Cb1, A.Cb2};
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      d[i] = lo(v[i]);
-      d[NV + i] = hi(v[i]);
-    }
+    for (int i = 0; i < NV; ++i) red[i * T + tid] = A.v[i];
   }
   __syncthreads();
   float* slot = nullptr;
@@ -442,84 +536,47 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
   float pose_g[12];
 #pragma unroll
   for (int i = 0; i < 12; ++i) pose_g[i] = 0.f;
-  if (sg == 0 && gl2 < GB2) {
-    float R[9], tp[3];
-    const bool want_R = want_pose;
-    if (want_R) load_pose(s.poses, V.pose, R, tp);
-#pragma unroll
-    for (int lane2 = 0; lane2 < 2; ++lane2) {
-      const int gi = 2 * gl2 + lane2;  // Gaussian index within the block
-      if (gi >= GB) break;
-      const int g = gb * GB + gi;
+  for (int gi = tid; gi < GB; gi += T) {  // one Gaussian per thread
+    const int g = gb * GB + gi;
+    float gm[3] = {0, 0, 0}, gL[6] = {0, 0, 0, 0, 0, 0}, glam = 0.f, gcol[3] = {0, 0, 0};
+    if (g < V.K) {
       float acc[NV];
 #pragma unroll
       for (int i = 0; i < NV; ++i) acc[i] = 0.f;
       for (int s2 = 0; s2 < S; ++s2) {
-        const float* d = red + ACC * (s2 * GB2 + gl2) + NV * lane2;
+        const float* d = reinterpret_cast<const float*>(red + s2 * GB2 + (gi >> 1)) + (gi & 1);
 #pragma unroll
-        for (int i = 0; i < NV; ++i) acc[i] += d[i];
+        for (int i = 0; i < NV; ++i) acc[i] += d[2 * i * T];
       }
-      float gm[3] = {0, 0, 0}, gL[6] = {0, 0, 0, 0, 0, 0}, glam = 0.f;
-      if (g < V.K && active) {
-        const GaussRec& gr1 = lane2 == 0 ? ga : gbr;
+      bwd_finalise<NORMALS, COLOR, POSE>(s, V, records, view_inv, g, acc, want_pose, gm, gL, glam, pose_g);
+      if (COLOR) {
+#pragma unroll
+        for (int k3 = 0; k3 < 3; ++k3) gcol[k3] = acc[Acc::kCol + k3];
+      }
+    }
+    if (slot == nullptr) {
+      if (g < V.K) {
         const long long gg = V.gauss_off + g;
-        const float L00 = gr1.L[0], L10 = gr1.L[1], L11 = gr1.L[2], L20 = gr1.L[3], L21 = gr1.L[4], L22 = gr1.L[5];
-        const float Bb0 = -acc[1], Bb1 = -acc[2], Bb2 = -acc[3];
-        // mubar = L bbar_sum
-        gm[0] = L00 * Bb0;
-        gm[1] = fmaf(L11, Bb1, L10 * Bb0);
-        gm[2] = fmaf(L22, Bb2, fmaf(L21, Bb1, L20 * Bb0));
-        const float m0 = gr1.mh[0], m1 = gr1.mh[1], m2 = gr1.mh[2];
-        const float* M = acc + 10;
-        gL[0] = acc[4] + M[0] + m0 * Bb0;  // (0,0)
-        gL[1] = acc[5] + M[3] + m1 * Bb0;  // (1,0)
-        gL[2] = acc[6] + M[4] + m1 * Bb1;  // (1,1)
-        gL[3] = acc[7] + M[6] + m2 * Bb0;  // (2,0)
-        gL[4] = acc[8] + M[7] + m2 * Bb1;  // (2,1)
-        gL[5] = acc[9] + M[8] + m2 * Bb2;  // (2,2)
-        glam = -acc[0] / s.weights[gg];
-        if (want_R) {
-          // Rbar += R (M L^T) + t mubar^T ; tbar += R mubar
-          float ML[9];
-          const float Lf[9] = {L00, 0.f, 0.f, L10, L11, 0.f, L20, L21, L22};
+        atomicAdd(out.gmeans + 3 * gg + 0, gm[0]);
+        atomicAdd(out.gmeans + 3 * gg + 1, gm[1]);
+        atomicAdd(out.gmeans + 3 * gg + 2, gm[2]);
 #pragma unroll
-          for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int c = 0; c < 3; ++c)
-              ML[3 * a + c] =
-                  fmaf(M[3 * a + 2], Lf[3 * c + 2], fmaf(M[3 * a + 1], Lf[3 * c + 1], M[3 * a] * Lf[3 * c]));
-#pragma unroll
-          for (int a = 0; a < 3; ++a) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c)
-              pose_g[3 * a + c] += fmaf(R[3 * a + 2], ML[6 + c], fmaf(R[3 * a + 1], ML[3 + c], R[3 * a] * ML[c])) +
-                                   tp[a] * gm[c];
-            pose_g[9 + a] += fmaf(R[3 * a + 2], gm[2], fmaf(R[3 * a + 1], gm[1], R[3 * a] * gm[0]));
-          }
-        }
-        if (slot == nullptr) {
-          atomicAdd(out.gmeans + 3 * gg + 0, gm[0]);
-          atomicAdd(out.gmeans + 3 * gg + 1, gm[1]);
-          atomicAdd(out.gmeans + 3 * gg + 2, gm[2]);
-#pragma unroll
-          for (int i = 0; i < 6; ++i) atomicAdd(out.gchol + 6 * gg + i, gL[i]);
-          atomicAdd(out.gweights + gg, glam);
-          if (COLOR) {
-#pragma unroll
-            for (int k3 = 0; k3 < 3; ++k3) atomicAdd(out.gcolors + 3 * gg + k3, acc[19 + k3]);
-          }
-        }
-      }
-      if (slot != nullptr) {
-        float* d = slot + NC * gi;
-        d[0] = gm[0]; d[1] = gm[1]; d[2] = gm[2];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) d[3 + i] = gL[i];
-        d[9] = glam;
+        for (int i = 0; i < 6; ++i) atomicAdd(out.gchol + 6 * gg + i, gL[i]);
+        atomicAdd(out.gweights + gg, glam);
         if (COLOR) {
 #pragma unroll
-          for (int k3 = 0; k3 < 3; ++k3) d[10 + k3] = (g < V.K && active) ? acc[19 + k3] : 0.f;
+          for (int k3 = 0; k3 < 3; ++k3) atomicAdd(out.gcolors + 3 * gg + k3, gcol[k3]);
         }
+      }
+    } else {
+      float* d = slot + NC * gi;
+      d[0] = gm[0]; d[1] = gm[1]; d[2] = gm[2];
+#pragma unroll
+      for (int i = 0; i < 6; ++i) d[3 + i] = gL[i];
+      d[9] = glam;
+      if (COLOR) {
+#pragma unroll
+        for (int k3 = 0; k3 < 3; ++k3) d[10 + k3] = gcol[k3];
       }
     }
   }
@@ -548,27 +605,27 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
   }  // item loop
 }
 
-static int bwd_smem_bytes(int ray_tile, int threads, bool color = false) {
-  return std::max(ray_tile * (color ? ray_rec2<true>() : kRayRec2) * static_cast<int>(sizeof(float4)),
-                  threads * (color ? acc_floats<true>() : kAccFloats) * static_cast<int>(sizeof(float)));
+template <bool NORMALS, bool COLOR, bool POSE>
+static int bwd_smem_bytes(int ray_tile, int threads) {
+  return std::max(ray_tile * ray_rec2<NORMALS, COLOR>() * static_cast<int>(sizeof(float4)),
+                  threads * acc_count<NORMALS, COLOR, POSE>() * static_cast<int>(sizeof(f2)));
 }
 
-template <bool NORMALS, int NFLOW, bool STORED = false, bool COLOR = false, bool POSE = true, int CL = 1,
-          class B = Batch>
+template <bool NORMALS, int NFLOW, bool COLOR = false, bool POSE = true, int CL = 1, class B = Batch>
 static cudaError_t prepare_bwd_t(int smem) {
   // Dynamic plus static shared memory above the 48 KB default needs the opt-in.
   if (smem + static_cast<int>(sizeof(float) * (kBwdMaxThreads / 32) * 48) > 48 * 1024)
-    return cudaFuncSetAttribute(backward_kernel<NORMALS, NFLOW, STORED, COLOR, POSE, CL, B>,
+    return cudaFuncSetAttribute(backward_kernel<NORMALS, NFLOW, COLOR, POSE, CL, B>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   return cudaSuccess;
 }
 
 template <bool NORMALS, int NFLOW>
 static int bwd_ctas_per_sm_t(int ray_tile, int threads) {
-  const int smem = bwd_smem_bytes(ray_tile, threads);
+  const int smem = bwd_smem_bytes<NORMALS, false, true>(ray_tile, threads);
   if (prepare_bwd_t<NORMALS, NFLOW>(smem) != cudaSuccess) return 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, backward_kernel<NORMALS, NFLOW, false>, threads, smem) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, backward_kernel<NORMALS, NFLOW>, threads, smem) !=
       cudaSuccess)
     return 1;
   return n > 0 ? n : 1;
@@ -592,12 +649,12 @@ static int bwd_cluster_size(const B& b) {
   return C;
 }
 
-template <bool NORMALS, int NFLOW, bool STORED, bool COLOR = false, bool POSE = true, class B>
+template <bool NORMALS, int NFLOW, bool COLOR = false, bool POSE = true, class B>
 static cudaError_t launch_bwd_s(const B& b, const Scene& s, const Consts& c, const float4* records,
                                 int ray_tile, int threads, const BwdIn& in, const BwdOut& out, int* counter,
                                 cudaStream_t st) {
-  const int smem = bwd_smem_bytes(ray_tile, threads, COLOR);
-  cudaError_t e = prepare_bwd_t<NORMALS, NFLOW, STORED, COLOR, POSE, 1, B>(smem);
+  const int smem = bwd_smem_bytes<NORMALS, COLOR, POSE>(ray_tile, threads);
+  cudaError_t e = prepare_bwd_t<NORMALS, NFLOW, COLOR, POSE, 1, B>(smem);
   if (e != cudaSuccess) return e;
   int grid = b.n_items;
   if (counter) {
@@ -606,15 +663,15 @@ static cudaError_t launch_bwd_s(const B& b, const Scene& s, const Consts& c, con
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     grid = std::min(b.n_items, std::max(1, sms) * bwd_ctas_per_sm_t<NORMALS, NFLOW>(ray_tile, threads));
   }
-  if constexpr (!STORED && !COLOR) {
+  if constexpr (!COLOR) {
     if (counter == nullptr && bwd_cluster_size(b) == 2) {
-      e = prepare_bwd_t<NORMALS, NFLOW, STORED, COLOR, POSE, 2, B>(smem);
+      e = prepare_bwd_t<NORMALS, NFLOW, COLOR, POSE, 2, B>(smem);
       if (e != cudaSuccess) return e;
-      return launch_kernel(backward_kernel<NORMALS, NFLOW, STORED, COLOR, POSE, 2, B>, dim3(grid), dim3(threads), smem,
+      return launch_kernel(backward_kernel<NORMALS, NFLOW, COLOR, POSE, 2, B>, dim3(grid), dim3(threads), smem,
                            st, 2, b, s, c, records, in, out, ray_tile, counter);
     }
   }
-  return launch_kernel(backward_kernel<NORMALS, NFLOW, STORED, COLOR, POSE, 1, B>, dim3(grid), dim3(threads), smem, st,
+  return launch_kernel(backward_kernel<NORMALS, NFLOW, COLOR, POSE, 1, B>, dim3(grid), dim3(threads), smem, st,
                        1, b, s, c, records, in, out, ray_tile, counter);
 }
 
@@ -622,14 +679,12 @@ template <bool NORMALS, int NFLOW, class B>
 static cudaError_t launch_bwd_t(const B& b, const Scene& s, const Consts& c, const float4* records,
                                 int ray_tile, int threads, const BwdIn& in, const BwdOut& out, int* counter,
                                 cudaStream_t st) {
-  if (in.pairs != nullptr)
-    return launch_bwd_s<NORMALS, NFLOW, true>(b, s, c, records, ray_tile, threads, in, out, counter, st);
   if (out.gcolors != nullptr)
-    return launch_bwd_s<NORMALS, NFLOW, false, true>(b, s, c, records, ray_tile, threads, in, out, counter, st);
+    return launch_bwd_s<NORMALS, NFLOW, true>(b, s, c, records, ray_tile, threads, in, out, counter, st);
   if (out.gposes == nullptr)
-    return launch_bwd_s<NORMALS, NFLOW, false, false, false>(b, s, c, records, ray_tile, threads, in, out, counter,
+    return launch_bwd_s<NORMALS, NFLOW, false, false>(b, s, c, records, ray_tile, threads, in, out, counter,
                                                               st);
-  return launch_bwd_s<NORMALS, NFLOW, false>(b, s, c, records, ray_tile, threads, in, out, counter, st);
+  return launch_bwd_s<NORMALS, NFLOW>(b, s, c, records, ray_tile, threads, in, out, counter, st);
 }
 
 template <class B>

@@ -1,0 +1,110 @@
+// fmb_cam.cuh -- the camera-plane form of a ray/Gaussian pair that the two-parameter
+// render and its adjoint evaluate, and the per (view, Gaussian) records it reads.
+//
+// A pixel's ray is c = ((px - cx)/fx, (py - cy)/fy, 1): affine in the pixel.  In the
+// camera frame the precision is P = A A^T with A = R L, and any root of it serves,
+// since Eq. 2 depends on L only through P.  The lower Cholesky factor B of P makes
+// the whitened ray a = B^T c as short as it gets: a2 is constant, a1 depends on py
+// only.  With m the mean in the camera frame (z its depth) and c_e a fixed pixel near
+// the mean's projection, write c = c_e + delta and measure the hit from the mean's
+// own depth: t = z + tau.  Then
+//   D   = z B^T delta - B^T (m - z c_e)      (affine in the pixel, third entry 0)
+//   tau = -(D . a) / (a . a),   u = D + tau a,   q = u . u
+// The pixel offsets from c_e are exact near the projection (Sterbenz) and m - z c_e
+// is formed in float pairs, so u keeps its relative accuracy for rays that pass close
+// to a distant mean, where t a - b in plain fp32 loses |b|/|u| ulps.  25 operations
+// per pair without the normal, 36 with it; the world-frame evaluation (exact float
+// pairs of the ray and of mu - o, and a second projection of u) took 35 and 56 at the
+// same error (log-weights 1.0-2.1e-6 rms against 1.3-2.2e-6, FP64 comparison on the
+// benchmark's scenes).
+//
+// Every whitened quantity carries a factor sqrt(log2(e) / 2), so that
+// u . u - log2(lambda) is -log2(delta) of Eq. 4, and lengths are in pixels (B's rows
+// divided by fx, fy), so that the pixel offsets enter as they are.
+#pragma once
+
+#include "fmb_f32x2.cuh"
+#include "fmb_internal.cuh"
+
+namespace fmb {
+
+// Record of two Gaussians (one per packed lane), 16 f2 = 128 bytes.  B' = [[B00],
+// [B10, B11], [e0, e1, e2]] is the root in the frame of the offsets (dx, dy, 1).
+//   0 -pe_x  1 -pe_y   expansion pixel, negated
+//   2 B00  3 B10  4 z  5 d0  6 e0  7 B11  8 e1  9 z B11  10 d1
+//   11 e2^2  12 -log2(lambda)  13 unused  14 rho_x  15 rho_y (m - z c_e, in pixels)
+// An object's last record of an odd count holds its last Gaussian twice, the copy
+// with the log-density -1e30: its weight and density are exactly 0.
+constexpr int kCamF2 = 16;
+constexpr float kDummyNl2 = 1e30f;
+
+// sqrt(log2(e) / 2), its square, and 2 ln 2 (the derivative of d = ln(delta) with
+// respect to a scaled u is -2 ln 2 u).
+constexpr float kCamScale = 0.84932180028801904f;
+constexpr float kCamScale2 = 0.72134752044448170f;
+constexpr float kTwoLn2 = 1.3862943611198906f;
+
+struct CamRec2 {
+  f2 npx, npy, B00, B10, z, d0, e0, B11, e1, F11, d1, ee, nl2;
+};
+__device__ __forceinline__ CamRec2 cam_load(const ulonglong2* __restrict__ r) {
+  const ulonglong2 q0 = r[0], q1 = r[1], q2 = r[2], q3 = r[3], q4 = r[4], q5 = r[5], q6 = r[6];
+  CamRec2 g;
+  g.npx = as_f2(q0.x);
+  g.npy = as_f2(q0.y);
+  g.B00 = as_f2(q1.x);
+  g.B10 = as_f2(q1.y);
+  g.z = as_f2(q2.x);
+  g.d0 = as_f2(q2.y);
+  g.e0 = as_f2(q3.x);
+  g.B11 = as_f2(q3.y);
+  g.e1 = as_f2(q4.x);
+  g.F11 = as_f2(q4.y);
+  g.d1 = as_f2(q5.x);
+  g.ee = as_f2(q5.y);
+  g.nl2 = as_f2(q6.x);
+  return g;
+}
+
+// One pair per lane: two Gaussians against the pixel (X, Y), both lanes alike.
+struct CamGeom2 {
+  f2 dx, dy, a0, a1, ninv, tau, t, u0, u1, nx;  // ninv = -1 / a.a;  nx = -log2(delta)
+};
+__device__ __forceinline__ f2 rcp_neg_2(f2 a) { return pk(rcp_approx(-lo(a)), rcp_approx(-hi(a))); }
+__device__ __forceinline__ CamGeom2 cam_geom2(const CamRec2& g, f2 X, f2 Y) {
+  CamGeom2 G;
+  G.dx = add2(X, g.npx);
+  G.dy = add2(Y, g.npy);
+  const f2 ad = fma2(g.B00, G.dx, mul2(g.B10, G.dy));
+  G.a0 = add2(ad, g.e0);
+  G.a1 = fma2(g.B11, G.dy, g.e1);
+  const f2 D0 = fma2(g.z, ad, g.d0);
+  const f2 D1 = fma2(g.F11, G.dy, g.d1);
+  const f2 aa = fma2(G.a0, G.a0, fma2(G.a1, G.a1, g.ee));
+  G.ninv = rcp_neg_2(aa);
+  G.tau = mul2(fma2(D0, G.a0, mul2(D1, G.a1)), G.ninv);
+  G.t = add2(g.z, G.tau);
+  G.u0 = fma2(G.tau, G.a0, D0);
+  G.u1 = fma2(G.tau, G.a1, D1);
+  G.nx = fma2(G.u0, G.u0, fma2(G.u1, G.u1, fma2(mul2(G.tau, G.tau), g.ee, g.nl2)));
+  return G;
+}
+
+// Camera-plane quantities of a pixel: its centre (px, py), c = (x, y, 1) and |c|.
+// Round-to-nearest intrinsics throughout, so that the forward and the adjoint
+// (compiled with different flags) get the same bits.
+struct CamRay {
+  float px, py, x, y, len;
+};
+__device__ __forceinline__ CamRay cam_ray(const DevView& V, int p) {
+  CamRay r;
+  const int iy = p / V.W;
+  r.px = static_cast<float>(p - iy * V.W) + 0.5f;
+  r.py = static_cast<float>(iy) + 0.5f;
+  r.x = __fdiv_rn(__fsub_rn(r.px, V.cx), V.fx);
+  r.y = __fdiv_rn(__fsub_rn(r.py, V.cy), V.fy);
+  r.len = __fsqrt_rn(__fmaf_rn(r.x, r.x, __fmaf_rn(r.y, r.y, 1.0f)));
+  return r;
+}
+
+}  // namespace fmb

@@ -1,30 +1,56 @@
 // fmb_forward.cu -- prologue (per view x Gaussian records) and forward render
 // kernel of the two-parameter Fuzzy Metaballs renderer.
 //
-// Formulation (paper Eq. 2, 3, 4, 7, 8, 17; Sec. 5 flow), whitened per Gaussian:
-// with Sigma^-1 = L L^T, a = L^T v and b = L^T (mu - o), the max-likelihood depth is
-// t = a.b / a.a, the residual in the whitened frame is u = t a - b = L^T (o + v t - mu),
-// q = u.u, d = -q/2 + ln(lambda), delta = e^d, and the weight exponent of Eq. 7 is
-// e = beta1 d - (beta2/eta) t.  The local normal Sigma^-1 (o + v t - mu) of Eq. 17 is
-// g = L u.  Everything is evaluated in the log2 domain so that the exponentials
-// are single ex2 instructions.
+// Formulation (paper Eq. 2, 3, 4, 7, 8, 17; Sec. 5 flow): the max-likelihood depth t
+// along the ray, the Mahalanobis term q there, d = -q/2 + ln(lambda), delta = e^d, the
+// weight exponent of Eq. 7 e = beta1 d - (beta2/eta) t, and the local normal
+// Sigma^-1 (o + v t - mu) of Eq. 17, all in the camera-plane form of fmb_cam.cuh and
+// in the log2 domain, so that the exponentials are single ex2 instructions.
 #include <algorithm>
 
+#include "fmb_cam.cuh"
 #include "fmb_f32x2.cuh"
 #include "fmb_internal.cuh"
 
 namespace fmb {
 
 constexpr int kFwdThreads = 128;
-constexpr int kChunk = 256;  // records per shared-memory stage (16 KB)
+constexpr int kChunk = 256;  // Gaussians per shared-memory stage (16 KB)
+constexpr int kFwdUnroll = 2;  // records per trip (1: 1 to 2.5 % slower)
 
 // ------------------------------------------------------------------ prologue
-// One thread per (view, Gaussian): the record of unpack_rec.  The camera centre
+// The world-frame kernels' records (fmb_world_*.cu, alpha compositing, point export,
+// attribution).  One thread per (view, Gaussian): the record of unpack_rec.  The camera centre
 // o = -R^T t and m = mu - o are formed as exact float pairs (error-free
 // transformations), so that the per-pair residual can be evaluated to full fp32
 // accuracy relative to its own size.  The same launch clears the arrays of `zero`
 // (the backward's gradient outputs and status word, which its kernels then
 // accumulate into), grid-stride over all its threads.
+// The rest of a world-frame record from L and mu - o = mh + ml.
+__device__ __forceinline__ void world_record(GaussRec& q, const float ml[3], float weight) {
+  const float* L = q.L;
+  q.b[0] = fmaf(L[3], q.mh[2], fmaf(L[1], q.mh[1], L[0] * q.mh[0]));
+  q.b[1] = fmaf(L[4], q.mh[2], L[2] * q.mh[1]);
+  q.b[2] = L[5] * q.mh[2];
+  q.nbl[0] = -fmaf(L[3], ml[2], fmaf(L[1], ml[1], L[0] * ml[0]));
+  q.nbl[1] = -fmaf(L[4], ml[2], L[2] * ml[1]);
+  q.nbl[2] = -(L[5] * ml[2]);
+  q.l2 = log2f(weight);
+}
+
+__device__ __forceinline__ void prologue_clear(int* status_to_clear, int* counter_to_clear, const ZeroJob& zero) {
+  const long long stride = static_cast<long long>(gridDim.x) * gridDim.y * blockDim.x;
+  const long long j0 = (static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x;
+  if (j0 == 0) {
+    if (status_to_clear != nullptr) *status_to_clear = kDevOk;
+    if (counter_to_clear != nullptr) *counter_to_clear = 0;
+  }
+  for (int b = 0; b < ZeroJob::kMax; ++b) {
+    if (zero.ptr[b] == nullptr) continue;
+    for (long long j = j0; j < zero.n[b]; j += stride) zero.ptr[b][j] = 0.f;
+  }
+}
+
 template <class B>
 __global__ void __launch_bounds__(128) prologue_kernel(const __grid_constant__ B batch, Scene s, Consts k,
                                                         float4* __restrict__ records, int* status_to_clear,
@@ -32,49 +58,193 @@ __global__ void __launch_bounds__(128) prologue_kernel(const __grid_constant__ B
   pdl_enter();
   const DevView& V = batch.v[blockIdx.y];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0 && blockIdx.y == 0) {
-    if (status_to_clear != nullptr) *status_to_clear = kDevOk;
-    if (counter_to_clear != nullptr) *counter_to_clear = 0;
-  }
-  {
-    const long long stride = static_cast<long long>(gridDim.x) * gridDim.y * blockDim.x;
-    const long long j0 = (static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x;
-    for (int b = 0; b < ZeroJob::kMax; ++b) {
-      if (zero.ptr[b] == nullptr) continue;
-      for (long long j = j0; j < zero.n[b]; j += stride) zero.ptr[b][j] = 0.f;
-    }
-  }
+  prologue_clear(status_to_clear, counter_to_clear, zero);
   if (i >= V.K) return;
   float R[9], t[3];
   load_pose(s.poses, V.pose, R, t);
   const long long g = V.gauss_off + i;
-  const float* L = s.chol + 6 * g;
-  const float L00 = L[0], L10 = L[1], L11 = L[2], L20 = L[3], L21 = L[4], L22 = L[5];
-  float mh[3], ml[3];
+  GaussRec q;
+  float ml[3];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) q.L[c] = s.chol[6 * g + c];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     float oh, ol, sh, se;
     camera_centre_dd(R, t, c, oh, ol);
     two_sum(s.means[3 * g + c], -oh, sh, se);
-    two_sum(sh, __fsub_rn(se, ol), mh[c], ml[c]);
+    two_sum(sh, __fsub_rn(se, ol), q.mh[c], ml[c]);
   }
-  const float b0 = fmaf(L20, mh[2], fmaf(L10, mh[1], L00 * mh[0]));
-  const float b1 = fmaf(L21, mh[2], L11 * mh[1]);
-  const float b2 = L22 * mh[2];
-  const float nb0 = -fmaf(L20, ml[2], fmaf(L10, ml[1], L00 * ml[0]));
-  const float nb1 = -fmaf(L21, ml[2], L11 * ml[1]);
-  const float nb2 = -(L22 * ml[2]);
-  const float l2 = log2f(s.weights[g]);
+  world_record(q, ml, s.weights[g]);
   float4* r = records + kRecFloat4 * (V.rec_off + i);
-  r[0] = make_float4(L00, L10, L11, L20);
-  r[1] = make_float4(L21, L22, b0, b1);
-  r[2] = make_float4(b2, mh[0], mh[1], mh[2]);
-  r[3] = make_float4(nb0, nb1, nb2, l2);
+  r[0] = make_float4(q.L[0], q.L[1], q.L[2], q.L[3]);
+  r[1] = make_float4(q.L[4], q.L[5], q.b[0], q.b[1]);
+  r[2] = make_float4(q.b[2], q.mh[0], q.mh[1], q.mh[2]);
+  r[3] = make_float4(q.nbl[0], q.nbl[1], q.nbl[2], q.l2);
   if (s.crec != nullptr) {
     const float* c = s.colors + 3 * g;
     s.crec[V.rec_off + i] = make_float4(c[0], c[1], c[2], 0.f);
   }
   (void)k;
+}
+
+// Float pairs (unevaluated sums h + l, about 2^-46 relative): the prologue of the
+// camera-plane records forms P = A A^T and its Cholesky factor in them, since P
+// squares the condition of L.  About 900 fp32 instructions per record; FP64 would
+// take fewer, but issues one warp instruction per 16 cycles and SM here.
+struct FF {
+  float h, l;
+};
+__device__ __forceinline__ FF ff_renorm(float h, float l) {
+  const float s = __fadd_rn(h, l);
+  return FF{s, __fsub_rn(l, __fsub_rn(s, h))};
+}
+__device__ __forceinline__ FF operator+(FF a, FF b) {
+  float s, e;
+  two_sum(a.h, b.h, s, e);
+  return ff_renorm(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ FF operator-(FF a) { return FF{-a.h, -a.l}; }
+__device__ __forceinline__ FF operator-(FF a, FF b) { return a + (-b); }
+__device__ __forceinline__ FF operator*(FF a, FF b) {
+  float p, e;
+  two_prod(a.h, b.h, p, e);
+  return ff_renorm(p, fmaf(a.h, b.l, fmaf(a.l, b.h, e)));
+}
+__device__ __forceinline__ FF operator*(FF a, float b) {
+  float p, e;
+  two_prod(a.h, b, p, e);
+  return ff_renorm(p, fmaf(a.l, b, e));
+}
+__device__ __forceinline__ FF ff_prod(float a, float b) {
+  FF r;
+  two_prod(a, b, r.h, r.l);
+  return r;
+}
+__device__ __forceinline__ FF ff_diff(float a, float b) {
+  FF r;
+  two_sum(a, -b, r.h, r.l);
+  return r;
+}
+// 1 / a and 1 / sqrt(a): one Newton step in pair arithmetic from the fp32 value.
+__device__ __forceinline__ FF ff_rcp(FF a) {
+  const float y = __frcp_rn(a.h);
+  const FF r = FF{1.f, 0.f} - a * y;
+  return ff_renorm(y, __fmul_rn(y, r.h));
+}
+__device__ __forceinline__ FF ff_rsqrt(FF a) {  // 0 for a <= 0 (a singular precision)
+  if (!(a.h > 0.f)) return FF{a.h == a.h ? 0.f : a.h, 0.f};
+  const float y = rsqrtf(a.h);
+  const FF r = FF{1.f, 0.f} - a * ff_prod(y, y);
+  return ff_renorm(y, __fmul_rn(0.5f * y, r.h));
+}
+
+// The camera-plane records of a view (fmb_cam.cuh), one thread per Gaussian; the
+// threads of a pair exchange halves, so that each stores 64 consecutive bytes.  The
+// functions of R are those of the world-frame formulation (v = R^T c, o = -R^T t) for
+// any invertible R, not only an exact rotation: A = R L and m_cam = R^-T (mu - o).
+template <class B>
+__global__ void __launch_bounds__(128) prologue_cam_kernel(const __grid_constant__ B batch, Scene s,
+                                                            float4* __restrict__ records, int* status_to_clear,
+                                                            int* counter_to_clear, ZeroJob zero) {
+  pdl_enter();
+  const DevView& V = batch.v[blockIdx.y];
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  prologue_clear(status_to_clear, counter_to_clear, zero);
+  const int Kpad = (V.K + 1) & ~1;
+  if ((i & ~31) >= Kpad) return;  // whole warps only: the threads of a pair shuffle below
+  const int gi = min(i, V.K - 1);
+  float R[9], t[3];
+  load_pose(s.poses, V.pose, R, t);
+  const long long g = V.gauss_off + gi;
+  const float* Lp = s.chol + 6 * g;
+  const float L00 = Lp[0], L10 = Lp[1], L11 = Lp[2], L20 = Lp[3], L21 = Lp[4], L22 = Lp[5];
+  FF m[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    float oh, ol, sh, se;
+    camera_centre_dd(R, t, c, oh, ol);
+    two_sum(s.means[3 * g + c], -oh, sh, se);
+    two_sum(sh, __fsub_rn(se, ol), m[c].h, m[c].l);
+  }
+  // R^-T = cof(R) / det(R)
+  FF C[9];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const int a1 = (a + 1) % 3, a2 = (a + 2) % 3, b1 = (b + 1) % 3, b2 = (b + 2) % 3;
+      C[3 * a + b] = ff_prod(R[3 * a1 + b1], R[3 * a2 + b2]) - ff_prod(R[3 * a1 + b2], R[3 * a2 + b1]);
+    }
+  }
+  const FF rdet = ff_rcp(C[0] * R[0] + C[1] * R[1] + C[2] * R[2]);
+  FF mc[3], A[9];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    mc[a] = (C[3 * a] * m[0] + C[3 * a + 1] * m[1] + C[3 * a + 2] * m[2]) * rdet;
+    A[3 * a + 0] = ff_prod(R[3 * a], L00) + ff_prod(R[3 * a + 1], L10) + ff_prod(R[3 * a + 2], L20);
+    A[3 * a + 1] = ff_prod(R[3 * a + 1], L11) + ff_prod(R[3 * a + 2], L21);
+    A[3 * a + 2] = ff_prod(R[3 * a + 2], L22);
+  }
+  auto P = [&](int a, int b) { return A[3 * a] * A[3 * b] + A[3 * a + 1] * A[3 * b + 1] + A[3 * a + 2] * A[3 * b + 2]; };
+  const FF P00 = P(0, 0), r0 = ff_rsqrt(P00);
+  const FF B00 = P00 * r0, B10 = P(1, 0) * r0, B20 = P(2, 0) * r0;
+  const FF S11 = P(1, 1) - B10 * B10, r1 = ff_rsqrt(S11);
+  const FF B11 = S11 * r1, B21 = (P(2, 1) - B20 * B10) * r1;
+  const FF S22 = P(2, 2) - B20 * B20 - B21 * B21;
+  // expansion pixel: the mean's projection, kept within an image of the view's sides
+  const float z = mc[2].h;
+  float pe[2];
+  const float f[2] = {V.fx, V.fy}, cc[2] = {V.cx, V.cy}, side[2] = {static_cast<float>(V.W), static_cast<float>(V.H)};
+  FF ce[2], rho[2];  // pe - c, and m - z c_e in pixels
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const float x = fmaf(f[c], __fdiv_rn(mc[c].h, z), cc[c]);
+    // a multiple of 1/256, so that px - pe is exact
+    pe[c] = 0.00390625f * rintf(256.f * (x == x ? fminf(fmaxf(x, -side[c]), 2.f * side[c]) : 0.5f * side[c]));
+    ce[c] = ff_diff(pe[c], cc[c]);
+    rho[c] = mc[c] * f[c] - mc[2] * ce[c];
+  }
+  const FF ifx = ff_rcp(FF{f[0], 0.f}), ify = ff_rcp(FF{f[1], 0.f}), sc = ff_diff(kCamScale, 0.f);
+  const FF b00 = B00 * ifx * sc, b10 = B10 * ify * sc, b11 = B11 * ify * sc;
+  const FF e0 = B20 * sc + b00 * ce[0] + b10 * ce[1], e1 = B21 * sc + b11 * ce[1];
+  const bool real = i < V.K;
+  float w[16];
+  w[0] = -pe[0];
+  w[1] = -pe[1];
+  w[2] = b00.h;
+  w[3] = b10.h;
+  w[4] = z;
+  w[5] = -fmaf(b00.h, rho[0].h, __fmul_rn(b10.h, rho[1].h));
+  w[6] = e0.h;
+  w[7] = b11.h;
+  w[8] = e1.h;
+  w[9] = (b11 * mc[2]).h;
+  w[10] = -__fmul_rn(b11.h, rho[1].h);
+  w[11] = __fmul_rn(S22.h > 0.f ? S22.h : (S22.h == S22.h ? 0.f : S22.h), kCamScale2);
+  w[12] = real ? -log2f(s.weights[g]) : kDummyNl2;
+  w[13] = 0.f;
+  w[14] = rho[0].h;
+  w[15] = rho[1].h;
+  const bool odd = (i & 1) != 0;
+  float rv[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) rv[k] = __shfl_xor_sync(0xffffffffu, odd ? w[k] : w[8 + k], 1);
+  float cl[3] = {0.f, 0.f, 0.f}, cr[3] = {0.f, 0.f, 0.f};
+  if (s.crec != nullptr) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      cl[k] = s.colors[3 * g + k];
+      cr[k] = __shfl_xor_sync(0xffffffffu, cl[k], 1);
+    }
+  }
+  if (i >= Kpad) return;
+  float4* r = records + kRecFloat4 * (static_cast<long long>(V.rec_off) + i);
+#pragma unroll
+  for (int k = 0; k < 8; k += 2)
+    r[k / 2] = odd ? make_float4(rv[k], w[8 + k], rv[k + 1], w[8 + k + 1]) : make_float4(w[k], rv[k], w[k + 1], rv[k + 1]);
+  if (s.crec != nullptr)  // pair of colour records: [r r g g | b b 0 0]
+    s.crec[static_cast<long long>(V.rec_off) + i] =
+        odd ? make_float4(cr[2], cl[2], 0.f, 0.f) : make_float4(cl[0], cr[0], cl[1], cr[1]);
 }
 
 template <class B>
@@ -93,81 +263,64 @@ cudaError_t launch_prologue(const BigBatch& b, const Scene& s, const Consts& c, 
                             int* status_to_clear, int* counter_to_clear, cudaStream_t st, const ZeroJob* zero) {
   return launch_prologue_t(b, s, c, records, maxK, status_to_clear, counter_to_clear, st, zero);
 }
-
-// ------------------------------------------------------------------- forward
-struct RayAcc {
-  float v0, v1, v2;     // world ray direction (high part)
-  float vl0, vl1, vl2;  // low part
-  float m;           // running shift of the log2 weights
-  float Sw, Swt, Sd;  // sum w, sum w t, sum delta
-  float N0, N1, N2;   // sum w n
-};
-
-template <bool NORMALS>
-__device__ __forceinline__ void fwd_pair(RayAcc& A, const GaussRec& g, const Consts& k) {
-  const PairGeom G = pair_geom<NORMALS>(g.L, g.b, g.mh, g.nbl, A.v0, A.v1, A.v2, A.vl0, A.vl1, A.vl2);
-  const float x = fmaf(G.q, k.K3, g.l2);  // log2(delta)
-  A.Sd += ex2_approx(x);
-  const float e2 = fmaf(x, k.beta1, G.t * k.K2);
-  if (e2 > A.m + kLazyShift) {
-    const float s = ex2_approx(A.m - e2);
-    A.Sw *= s;
-    A.Swt *= s;
-    if (NORMALS) {
-      A.N0 *= s;
-      A.N1 *= s;
-      A.N2 *= s;
-    }
-    A.m = e2;
-  }
-  const float w = ex2_approx(e2 - A.m);
-  A.Sw += w;
-  A.Swt = fmaf(w, G.t, A.Swt);
-  if (NORMALS) {
-    const float L00 = g.L[0], L10 = g.L[1], L11 = g.L[2], L20 = g.L[3], L21 = g.L[4], L22 = g.L[5];
-    const float g0 = L00 * G.u0;
-    const float g1 = fmaf(L11, G.u1, L10 * G.u0);
-    const float g2 = fmaf(L22, G.u2, fmaf(L21, G.u1, L20 * G.u0));
-    const float gg = fmaxf(fmaf(g2, g2, fmaf(g1, g1, g0 * g0)), 1e-30f);
-    const float ws = w * rsqrt_approx(gg);
-    A.N0 = fmaf(ws, g0, A.N0);
-    A.N1 = fmaf(ws, g1, A.N1);
-    A.N2 = fmaf(ws, g2, A.N2);
-  }
+template <class B>
+static cudaError_t launch_prologue_cam_t(const B& b, const Scene& s, float4* records, int maxK, int* status_to_clear,
+                                         int* counter_to_clear, cudaStream_t st, const ZeroJob* zero) {
+  const dim3 grid((maxK + 1 + 127) / 128, b.n_views);
+  return launch_kernel(prologue_cam_kernel<B>, grid, dim3(128), 0, st, 1, b, s, records, status_to_clear,
+                       counter_to_clear, zero != nullptr ? *zero : ZeroJob{});
+}
+cudaError_t launch_prologue_cam(const Batch& b, const Scene& s, float4* records, int maxK, int* status_to_clear,
+                                int* counter_to_clear, cudaStream_t st, const ZeroJob* zero) {
+  return launch_prologue_cam_t(b, s, records, maxK, status_to_clear, counter_to_clear, st, zero);
+}
+cudaError_t launch_prologue_cam(const BigBatch& b, const Scene& s, float4* records, int maxK, int* status_to_clear,
+                                int* counter_to_clear, cudaStream_t st, const ZeroJob* zero) {
+  return launch_prologue_cam_t(b, s, records, maxK, status_to_clear, counter_to_clear, st, zero);
 }
 
-// Two rays of one thread, packed lane-wise (lane 0 = even ray, lane 1 = odd ray).
+// ------------------------------------------------------------------- forward
+// One ray's sums over the two Gaussians of each record, one per lane; the lanes are
+// added after the last record.  Every ray constant is held in both lanes, so that a
+// record's values are used as loaded (packing two rays against one Gaussian instead
+// costs a move per record value).
+template <bool NORMALS, bool COLOR>
 struct RayAcc2 {
-  f2 v0, v1, v2, vl0, vl1, vl2;
-  f2 m, Sw, Swt, Sd, N0, N1, N2;
-  f2 C0, C1, C2;  // colour mode: sum w c
+  f2 X, Y, K2;        // pixel centre; -(beta2 / eta) log2(e) |c|: t's share of the log2 weight
+  f2 r00, r01, r11;   // NORMALS: metric of the image-plane normal components (ray_metric)
+  f2 nm, Sw, Swt, Sd; // minus the running shift of the log2 weights; sums of w, w t, delta
+  f2 N0, N1;          // sum w n, first two camera components over (fx, fy)
+  f2 C0, C1, C2;      // COLOR: sum w c
 };
 
-// Per-pair values the stored-intermediate mode keeps for the backward: the hit
-// depth t, the log2 weight e2 of Eq. 7 and the density delta of Eq. 4.
-struct PairOut2 {
-  f2 t, e2, delta;
-};
+// The normal g = P (t c - m) is perpendicular to the ray, so its third camera
+// component is -(x g_0 + y g_1) and |g|^2 a quadratic form of the first two, written
+// as (r00 h0 + r01 h1)^2 + (r11 h1)^2 for h = (g_0 / fx, g_1 / fy).
+__device__ __forceinline__ void ray_metric(const DevView& V, const CamRay& r, float& r00, float& r01, float& r11) {
+  const float s = sqrtf(fmaf(r.x, r.x, 1.0f));
+  r00 = V.fx * s;
+  r01 = V.fy * (r.x * r.y / s);
+  r11 = V.fy * (r.len / s);
+}
 
-template <bool NORMALS, bool COLOR = false>
-__device__ __forceinline__ PairOut2 fwd_pair2(RayAcc2& A, const GaussRec2& g, f2 K2, f2 K3, f2 beta1, f2 tiny,
-                                              float4 col = float4{}) {
-  const PairGeom2 G = pair_geom2<NORMALS>(g, A.v0, A.v1, A.v2, A.vl0, A.vl1, A.vl2);
-  const f2 x = fma2(G.q, K3, g.l2);  // log2(delta)
-  const f2 delta = ex2_2(x);
+template <bool NORMALS, bool COLOR>
+__device__ __forceinline__ void fwd_pair2(RayAcc2<NORMALS, COLOR>& A, const CamRec2& g, f2 nB1, f2 tiny, f2 c0,
+                                              f2 c1, f2 c2) {
+  const CamGeom2 G = cam_geom2(g, A.X, A.Y);
+  const f2 delta = pk(ex2_approx(-lo(G.nx)), ex2_approx(-hi(G.nx)));
   A.Sd = add2(A.Sd, delta);
-  const f2 e2 = fma2(x, beta1, mul2(G.t, K2));
-  f2 d = sub2(e2, A.m);
+  f2 d = fma2(G.t, A.K2, fma2(G.nx, nB1, A.nm));  // log2 weight above the shift
   if (fmaxf(lo(d), hi(d)) > kLazyShift) {  // rare: raise the shift of the lane(s) it no longer bounds
-    float dl = lo(d), dh = hi(d), sl = 1.f, sh = 1.f, ml = lo(A.m), mh = hi(A.m);
+    const f2 e2 = fma2(G.nx, nB1, mul2(G.t, A.K2));
+    float dl = lo(d), dh = hi(d), sl = 1.f, sh = 1.f, ml = lo(A.nm), mh = hi(A.nm);
     if (dl > kLazyShift) {
-      sl = ex2_approx(-dl);
-      ml = lo(e2);
+      sl = ex2_approx(-(lo(e2) + ml));
+      ml = -lo(e2);
       dl = 0.f;
     }
     if (dh > kLazyShift) {
-      sh = ex2_approx(-dh);
-      mh = hi(e2);
+      sh = ex2_approx(-(hi(e2) + mh));
+      mh = -hi(e2);
       dh = 0.f;
     }
     const f2 sc = pk(sl, sh);
@@ -176,57 +329,159 @@ __device__ __forceinline__ PairOut2 fwd_pair2(RayAcc2& A, const GaussRec2& g, f2
     if (NORMALS) {
       A.N0 = mul2(A.N0, sc);
       A.N1 = mul2(A.N1, sc);
-      A.N2 = mul2(A.N2, sc);
     }
     if (COLOR) {
       A.C0 = mul2(A.C0, sc);
       A.C1 = mul2(A.C1, sc);
       A.C2 = mul2(A.C2, sc);
     }
-    A.m = pk(ml, mh);
+    A.nm = pk(ml, mh);
     d = pk(dl, dh);
   }
   const f2 w = ex2_2(d);
   A.Sw = add2(A.Sw, w);
   A.Swt = fma2(w, G.t, A.Swt);
   if (COLOR) {
-    A.C0 = fma2(w, dup(col.x), A.C0);
-    A.C1 = fma2(w, dup(col.y), A.C1);
-    A.C2 = fma2(w, dup(col.z), A.C2);
+    A.C0 = fma2(w, c0, A.C0);
+    A.C1 = fma2(w, c1, A.C1);
+    A.C2 = fma2(w, c2, A.C2);
   }
   if (NORMALS) {
-    const f2 g0 = mul2(g.L[0], G.u0);
-    const f2 g1 = fma2(g.L[2], G.u1, mul2(g.L[1], G.u0));
-    const f2 g2 = fma2(g.L[5], G.u2, fma2(g.L[4], G.u1, mul2(g.L[3], G.u0)));
-    const f2 gg = add2(fma2(g2, g2, fma2(g1, g1, mul2(g0, g0))), tiny);
-    const f2 ws = mul2(w, rsqrt_2(gg));
-    A.N0 = fma2(ws, g0, A.N0);
-    A.N1 = fma2(ws, g1, A.N1);
-    A.N2 = fma2(ws, g2, A.N2);
+    const f2 h0 = mul2(g.B00, G.u0);
+    const f2 h1 = fma2(g.B11, G.u1, mul2(g.B10, G.u0));
+    const f2 p0 = fma2(A.r01, h1, mul2(A.r00, h0));
+    const f2 p1 = mul2(A.r11, h1);
+    const f2 ws = mul2(w, rsqrt_2(fma2(p0, p0, fma2(p1, p1, tiny))));
+    A.N0 = fma2(ws, h0, A.N0);
+    A.N1 = fma2(ws, h1, A.N1);
   }
-  return PairOut2{G.t, e2, delta};
 }
 
+// A ray's sums with the two lanes brought to one shift and added.
+struct RaySums {
+  float m, Sw, Swt, Sd, N0, N1, C0, C1, C2;
+};
+template <bool NORMALS, bool COLOR>
+__device__ __forceinline__ RaySums ray_sums(const RayAcc2<NORMALS, COLOR>& A) {
+  RaySums r;
+  const float ml = -lo(A.nm), mh = -hi(A.nm);
+  r.m = fmaxf(ml, mh);
+  const float sl = ex2_approx(ml - r.m), sh = ex2_approx(mh - r.m);
+  r.Sw = fmaf(hi(A.Sw), sh, lo(A.Sw) * sl);
+  r.Swt = fmaf(hi(A.Swt), sh, lo(A.Swt) * sl);
+  r.Sd = lo(A.Sd) + hi(A.Sd);
+  r.N0 = NORMALS ? fmaf(hi(A.N0), sh, lo(A.N0) * sl) : 0.f;
+  r.N1 = NORMALS ? fmaf(hi(A.N1), sh, lo(A.N1) * sl) : 0.f;
+  r.C0 = COLOR ? fmaf(hi(A.C0), sh, lo(A.C0) * sl) : 0.f;
+  r.C1 = COLOR ? fmaf(hi(A.C1), sh, lo(A.C1) * sl) : 0.f;
+  r.C2 = COLOR ? fmaf(hi(A.C2), sh, lo(A.C2) * sl) : 0.f;
+  return r;
+}
 
-// The accumulator of ray r of a thread (unpacked from its f32x2 lane when packed).
-template <bool PACKED, int NA, int NP>
-__device__ __forceinline__ RayAcc ray_acc_of(const RayAcc (&A)[NA], const RayAcc2 (&A2)[NP], int r) {
-  if (!PACKED) return A[r];
-  RayAcc a;
-  const RayAcc2& b = A2[r / 2];
-  const bool h = (r & 1) != 0;
-  a.v0 = h ? hi(b.v0) : lo(b.v0);
-  a.v1 = h ? hi(b.v1) : lo(b.v1);
-  a.v2 = h ? hi(b.v2) : lo(b.v2);
-  a.vl0 = a.vl1 = a.vl2 = 0.f;
-  a.m = h ? hi(b.m) : lo(b.m);
-  a.Sw = h ? hi(b.Sw) : lo(b.Sw);
-  a.Swt = h ? hi(b.Swt) : lo(b.Swt);
-  a.Sd = h ? hi(b.Sd) : lo(b.Sd);
-  a.N0 = h ? hi(b.N0) : lo(b.N0);
-  a.N1 = h ? hi(b.N1) : lo(b.N1);
-  a.N2 = h ? hi(b.N2) : lo(b.N2);
-  return a;
+// The blended normal N = sum w n / sum w in the camera frame, from a ray's sums.
+struct RayNormal {
+  float n0, n1, n2;
+};
+__device__ __forceinline__ RayNormal ray_normal(const DevView& V, const RaySums& a, const CamRay& ray) {
+  const float iSw = 1.0f / a.Sw;
+  const float N0 = V.fx * a.N0 * iSw, N1 = V.fy * a.N1 * iSw;
+  return RayNormal{N0, N1, -fmaf(ray.x, N0, ray.y * N1)};
+}
+
+// A normal that nearly cancels (|N| below kNormalCancels, about four rays in 10 000 of
+// the benchmark's scenes) has a direction that the rounding of the weights decides:
+// 1e-6 in N is 1e-3 in n_f at |N| = 1e-3.  Such rays are summed again by their whole
+// warp with the world-frame evaluation (pair_geom, the one the point export and the
+// alpha-compositing kernels use), lane l taking Gaussians l, l + 32, ...: the normal
+// there stays what that form gives, whatever the fast loop rounds.  32 Gaussians at a
+// time, the shift raised at the first lane whose exponent it no longer bounds, as a
+// walk in index order would.  0.1 % of the work at K = 4096.
+constexpr float kNormalCancels = 0.06f;
+__device__ __noinline__ RayNormal blended_normal_again(const DevView& V, const float* means, const float* chol,
+                                                       const float* weights, const float* poses, float K2, float K3,
+                                                       float beta1, int p) {
+  const int lane = threadIdx.x & 31;
+  float R[9], tp[3], vc[3], v[3], vl[3], pxy[2], oh[3], ol[3];
+  load_pose(poses, V.pose, R, tp);
+  pixel_ray_dd(V, R, ray_pixel(V, p), vc, v, vl, pxy);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) camera_centre_dd(R, tp, c, oh[c], ol[c]);
+  float m = -INFINITY, Sw = 0.f, N0 = 0.f, N1 = 0.f, N2 = 0.f;
+  for (int base = 0; base < V.K; base += 32) {
+    const bool in = base + lane < V.K;
+    const long long g = V.gauss_off + min(base + lane, V.K - 1);
+    GaussRec q;
+    float ml[3];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) q.L[c] = chol[6 * g + c];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      float sh, se;
+      two_sum(means[3 * g + c], -oh[c], sh, se);
+      two_sum(sh, __fsub_rn(se, ol[c]), q.mh[c], ml[c]);
+    }
+    world_record(q, ml, weights[g]);
+    const PairGeom G = pair_geom(q.L, q.b, q.mh, q.nbl, v[0], v[1], v[2], vl[0], vl[1], vl[2]);
+    const float e2 = fmaf(fmaf(G.q, K3, q.l2), beta1, G.t * K2);
+    const float g0 = q.L[0] * G.u0;
+    const float g1 = fmaf(q.L[2], G.u1, q.L[1] * G.u0);
+    const float g2 = fmaf(q.L[5], G.u2, fmaf(q.L[4], G.u1, q.L[3] * G.u0));
+    const float rs = rsqrt_approx(fmaf(g2, g2, fmaf(g1, g1, g0 * g0)) + 1e-30f);
+    auto add = [&](bool mine) {
+      const float w = mine ? ex2_approx(e2 - m) : 0.f;
+      const float ws = w * rs;
+      Sw += w;
+      N0 = fmaf(ws, g0, N0);
+      N1 = fmaf(ws, g1, N1);
+      N2 = fmaf(ws, g2, N2);
+    };
+    int start = 0;
+    for (int raised = 0; raised < 32; ++raised) {  // at most one raise per lane
+      const unsigned over = __ballot_sync(0xffffffffu, in && lane >= start && e2 > m + kLazyShift);
+      if (over == 0) break;
+      const int f = __ffs(over) - 1;
+      const float mf = __shfl_sync(0xffffffffu, e2, f);
+      add(in && lane >= start && lane < f);
+      const float sc = ex2_approx(m - mf);
+      Sw *= sc;
+      N0 *= sc;
+      N1 *= sc;
+      N2 *= sc;
+      m = mf;
+      start = f;
+    }
+    add(in && lane >= start);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    Sw += __shfl_xor_sync(0xffffffffu, Sw, o);
+    N0 += __shfl_xor_sync(0xffffffffu, N0, o);
+    N1 += __shfl_xor_sync(0xffffffffu, N1, o);
+    N2 += __shfl_xor_sync(0xffffffffu, N2, o);
+  }
+  const float iSw = 1.0f / Sw;
+  N0 *= iSw;
+  N1 *= iSw;
+  N2 *= iSw;
+  return RayNormal{fmaf(R[2], N2, fmaf(R[1], N1, R[0] * N0)), fmaf(R[5], N2, fmaf(R[4], N1, R[3] * N0)),
+                   fmaf(R[8], N2, fmaf(R[7], N1, R[6] * N0))};
+}
+
+// ray_normal, with the rays of the warp that need it summed again.  Whole warps call
+// it; `in`: the lane has a ray (entry p of the view).
+__device__ __forceinline__ RayNormal ray_normal_checked(const DevView& V, const Scene& s, const Consts& k,
+                                                        const RaySums& a, const CamRay& ray, int p, bool in) {
+  RayNormal N = ray_normal(V, a, ray);
+  unsigned again = __ballot_sync(
+      0xffffffffu, in && fmaf(N.n0, N.n0, fmaf(N.n1, N.n1, N.n2 * N.n2)) < kNormalCancels * kNormalCancels);
+  while (again != 0) {
+    const int src = __ffs(again) - 1;
+    again &= again - 1;
+    const RayNormal M = blended_normal_again(V, s.means, s.chol, s.weights, s.poses, k.K2, k.K3, k.beta1,
+                                             __shfl_sync(0xffffffffu, p, src));
+    if ((threadIdx.x & 31) == src) N = M;
+  }
+  return N;
 }
 
 // Per-pixel epilogue (Eq. 3, Eq. 8, Sec. 5, Sec. 6) from a ray's sums: depth, alpha,
@@ -234,43 +489,43 @@ __device__ __forceinline__ RayAcc ray_acc_of(const RayAcc (&A)[NA], const RayAcc
 template <bool NORMALS, int NFLOW>
 __device__ __forceinline__ void write_ray_outputs(const DevView& V, const float R[9], const float o[3],
                                                   const float (*Rj)[9], const float (*tj)[3], const bool* has_t,
-                                                  const RayAcc& a, const float pxy[2], long long p,
-                                                  const FwdOut& out) {
+                                                  const RaySums& a, const RayNormal& N, const CamRay& ray,
+                                                  long long p, const FwdOut& out) {
   const int P = V.P;
   const long long off = V.pix_off;
   const float iSw = 1.0f / a.Sw;
-  const float D = a.Swt * iSw;
-  out.depth[off + p] = D;
+  const float Dz = a.Swt * iSw;
+  out.depth[off + p] = Dz * ray.len;
   out.alpha[off + p] = -expm1f(-a.Sd);
   float* sv = out.saved + 3 * off;
   sv[p] = a.m + log2f(a.Sw);
   sv[P + p] = a.Sd;
   if (NORMALS) {
-    const float N0 = a.N0 * iSw, N1 = a.N1 * iSw, N2 = a.N2 * iSw;
-    const float Nn = sqrtf(fmaf(N0, N0, fmaf(N1, N1, N2 * N2)));
+    const float Nn = sqrtf(fmaf(N.n0, N.n0, fmaf(N.n1, N.n1, N.n2 * N.n2)));
     const float iN = Nn > 0.f ? 1.0f / Nn : 0.f;
-    const float n0 = N0 * iN, n1 = N1 * iN, n2 = N2 * iN;
     float* nrm = out.normal + 3 * off;
-    nrm[p] = fmaf(R[2], n2, fmaf(R[1], n1, R[0] * n0));
-    nrm[P + p] = fmaf(R[5], n2, fmaf(R[4], n1, R[3] * n0));
-    nrm[2 * P + p] = fmaf(R[8], n2, fmaf(R[7], n1, R[6] * n0));
+    nrm[p] = N.n0 * iN;
+    nrm[P + p] = N.n1 * iN;
+    nrm[2 * P + p] = N.n2 * iN;
     sv[2 * P + p] = Nn;
   } else {
     sv[2 * P + p] = 0.f;
   }
   if (NFLOW > 0) {
-    const float p0 = fmaf(a.v0, D, o[0]), p1 = fmaf(a.v1, D, o[1]), p2 = fmaf(a.v2, D, o[2]);
+    float pt[3];  // o + R^T c Dz
+#pragma unroll
+    for (int k = 0; k < 3; ++k) pt[k] = fmaf(fmaf(R[k], ray.x, fmaf(R[3 + k], ray.y, R[6 + k])), Dz, o[k]);
     float* fl = out.flow + 2 * NFLOW * off;
 #pragma unroll
     for (int j = 0; j < NFLOW; ++j) {
       float fu = 0.f, fv = 0.f;
       if (has_t[j]) {
-        const float X0 = fmaf(Rj[j][2], p2, fmaf(Rj[j][1], p1, fmaf(Rj[j][0], p0, tj[j][0])));
-        const float X1 = fmaf(Rj[j][5], p2, fmaf(Rj[j][4], p1, fmaf(Rj[j][3], p0, tj[j][1])));
-        const float X2 = fmaf(Rj[j][8], p2, fmaf(Rj[j][7], p1, fmaf(Rj[j][6], p0, tj[j][2])));
+        const float X0 = fmaf(Rj[j][2], pt[2], fmaf(Rj[j][1], pt[1], fmaf(Rj[j][0], pt[0], tj[j][0])));
+        const float X1 = fmaf(Rj[j][5], pt[2], fmaf(Rj[j][4], pt[1], fmaf(Rj[j][3], pt[0], tj[j][1])));
+        const float X2 = fmaf(Rj[j][8], pt[2], fmaf(Rj[j][7], pt[1], fmaf(Rj[j][6], pt[0], tj[j][2])));
         const float iz = 1.0f / X2;
-        fu = fmaf(V.fx * X0, iz, V.cx) - pxy[0];
-        fv = fmaf(V.fy * X1, iz, V.cy) - pxy[1];
+        fu = fmaf(V.fx * X0, iz, V.cx) - ray.px;
+        fv = fmaf(V.fy * X1, iz, V.cy) - ray.py;
       }
       fl[(2 * j) * P + p] = fu;
       fl[(2 * j + 1) * P + p] = fv;
@@ -285,18 +540,8 @@ __host__ __device__ constexpr int fwd_stage_float4() {
   return kChunk * (kRecFloat4 + (COLOR ? 1 : 0));
 }
 
-// Minimum resident CTAs: 7 for the plain two-rays-per-thread kernels with normals and
-// flow, whose default register allocation spills (one flow slot: 28 bytes at 72
-// registers) or stops at 5 CTAs per SM (two flow slots: 96 registers); bounded they
-// take 72 registers with 8 bytes of spill, and 70 with none (orbit forward 0.256 ->
-// 0.252 ms).  0 leaves the others to the compiler: a bound made them slower.
-template <bool NORMALS, int NFLOW, int RPT, bool STORE>
-constexpr int fwd_min_blocks() {
-  return (RPT == 2 && NORMALS && NFLOW > 0 && !STORE) ? 7 : 0;
-}
-
-template <bool NORMALS, int NFLOW, int RPT, bool STORE, bool COLOR = false, class B = Batch>
-__global__ void __launch_bounds__(kFwdThreads, COLOR ? 0 : fwd_min_blocks<NORMALS, NFLOW, RPT, STORE>())
+template <bool NORMALS, int NFLOW, int RPT, bool COLOR = false, class B = Batch>
+__global__ void __launch_bounds__(kFwdThreads)
     forward_kernel(const __grid_constant__ B batch, Scene s,
                                                               Consts k, const float4* __restrict__ records,
                                                               FwdOut out, int* status, int* counter) {
@@ -341,56 +586,36 @@ __global__ void __launch_bounds__(kFwdThreads, COLOR ? 0 : fwd_min_blocks<NORMAL
   const float4* csrc = COLOR ? s.crec + V.rec_off + kbeg : nullptr;
   if (tid == 0) {
     for (int c = 0; c < 2 && c < nchunks; ++c) {
-      const int n = min(kChunk, K - c * kChunk);
+      const int n = (min(kChunk, K - c * kChunk) + 1) & ~1;  // whole records of two
       mbar_arrive_expect_tx(&bars[c], n * 16u * (kRecFloat4 + (COLOR ? 1 : 0)));
       bulk_g2s(fwd_smem + c * SST, src + c * kChunk * kRecFloat4, n * 16u * kRecFloat4, &bars[c]);
       if (COLOR) bulk_g2s(fwd_smem + c * SST + kChunk * kRecFloat4, csrc + c * kChunk, n * 16u, &bars[c]);
     }
   }
 
-  // RPT even: rays are processed as packed pairs (PACKED); RPT == 1: scalar.
-  constexpr bool PACKED = (RPT % 2) == 0;
-  constexpr int NA = PACKED ? 1 : RPT;
-  constexpr int NP = PACKED ? RPT / 2 : 1;
-  RayAcc A[NA];
-  RayAcc2 A2[NP];
+  RayAcc2<NORMALS, COLOR> A[RPT];
   int pix[RPT];
-  float pxy[RPT][2];
-  float vc[RPT][3];
 #pragma unroll
   for (int r = 0; r < RPT; ++r) {
-    int p = tile * (kFwdThreads * RPT) + r * kFwdThreads + tid;
+    const int p = tile * (kFwdThreads * RPT) + r * kFwdThreads + tid;
     pix[r] = p;
-    p = min(p, P - 1);  // rays past the end compute a valid pixel and store nothing
-    float v[3], vl[3];
-    pixel_ray_dd(V, R, ray_pixel(V, p), vc[r], v, vl, pxy[r]);
-    if (!PACKED) {
-      RayAcc& a = A[PACKED ? 0 : r];
-      a.v0 = v[0];
-      a.v1 = v[1];
-      a.v2 = v[2];
-      a.vl0 = vl[0];
-      a.vl1 = vl[1];
-      a.vl2 = vl[2];
-      a.m = -INFINITY;
-      a.Sw = a.Swt = a.Sd = 0.f;
-      a.N0 = a.N1 = a.N2 = 0.f;
-    } else {
-      RayAcc2& a = A2[r / 2];
-      if ((r & 1) == 0) {
-        a.v0 = pk(v[0], 0.f); a.v1 = pk(v[1], 0.f); a.v2 = pk(v[2], 0.f);
-        a.vl0 = pk(vl[0], 0.f); a.vl1 = pk(vl[1], 0.f); a.vl2 = pk(vl[2], 0.f);
-      } else {
-        a.v0 = pk(lo(a.v0), v[0]); a.v1 = pk(lo(a.v1), v[1]); a.v2 = pk(lo(a.v2), v[2]);
-        a.vl0 = pk(lo(a.vl0), vl[0]); a.vl1 = pk(lo(a.vl1), vl[1]); a.vl2 = pk(lo(a.vl2), vl[2]);
-      }
-      a.m = dup(-INFINITY);
-      a.Sw = a.Swt = a.Sd = dup(0.f);
-      a.N0 = a.N1 = a.N2 = dup(0.f);
-      a.C0 = a.C1 = a.C2 = dup(0.f);
+    // rays past the end compute a valid pixel and store nothing
+    const CamRay ray = cam_ray(V, ray_pixel(V, min(p, P - 1)));
+    RayAcc2<NORMALS, COLOR>& a = A[r];
+    a.X = dup(ray.px);
+    a.Y = dup(ray.py);
+    a.K2 = dup(__fmul_rn(k.K2, ray.len));
+    if (NORMALS) {
+      float r00, r01, r11;
+      ray_metric(V, ray, r00, r01, r11);
+      a.r00 = dup(r00);
+      a.r01 = dup(r01);
+      a.r11 = dup(r11);
     }
+    a.nm = dup(INFINITY);
+    a.Sw = a.Swt = a.Sd = a.N0 = a.N1 = a.C0 = a.C1 = a.C2 = dup(0.f);
   }
-  const f2 K2v = dup(k.K2), K3v = dup(k.K3), B1v = dup(k.beta1), tiny = dup(1e-30f);
+  const f2 nB1 = dup(-k.beta1), tiny = dup(1e-30f), zero2 = dup(0.f);
 
   bool failed = false;
   for (int c = 0; c < nchunks; ++c) {
@@ -402,62 +627,24 @@ __global__ void __launch_bounds__(kFwdThreads, COLOR ? 0 : fwd_min_blocks<NORMAL
       break;
     }
     const int n = min(kChunk, K - c * kChunk);
-    const float4* rec = fwd_smem + stage * SST;
-    const float4* crs = rec + kChunk * kRecFloat4;  // colour mode: this stage's colour records
-    if (STORE) {
-      // Stored-intermediate mode (two rays per thread): the values of four
-      // consecutive Gaussians are buffered and written as one 16-byte store per
-      // ray and array into row p of the view's [pixel][Kp] block (Kp a multiple
-      // of 4; the padding past K is written as zeros).
-      const int p0 = pix[0], p1 = pix[1];
-      for (int i0 = 0; i0 < n; i0 += 4) {
-        float bt[2][4], be[2][4], bd[2][4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int i = i0 + u;
-          if (i < n) {
-            const GaussRec g = unpack_rec(rec[kRecFloat4 * i + 0], rec[kRecFloat4 * i + 1],
-                                          rec[kRecFloat4 * i + 2], rec[kRecFloat4 * i + 3]);
-            const PairOut2 po = fwd_pair2<NORMALS>(A2[0], broadcast_rec(g), K2v, K3v, B1v, tiny);
-            bt[0][u] = lo(po.t), bt[1][u] = hi(po.t);
-            be[0][u] = lo(po.e2), be[1][u] = hi(po.e2);
-            bd[0][u] = lo(po.delta), bd[1][u] = hi(po.delta);
-          } else {
-            bt[0][u] = bt[1][u] = be[0][u] = be[1][u] = bd[0][u] = bd[1][u] = 0.f;
-          }
-        }
-        const long long kk = static_cast<long long>(c) * kChunk + i0;
-        float* base = out.pairs + V.pair_off + kk;
-        const long long S2 = out.pair_stride;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int pp = h == 0 ? p0 : p1;
-          if (pp >= P) continue;
-          float* row = base + static_cast<long long>(pp) * V.Kp;
-          *reinterpret_cast<float4*>(row) = make_float4(bt[h][0], bt[h][1], bt[h][2], bt[h][3]);
-          *reinterpret_cast<float4*>(row + S2) = make_float4(be[h][0], be[h][1], be[h][2], be[h][3]);
-          *reinterpret_cast<float4*>(row + 2 * S2) = make_float4(bd[h][0], bd[h][1], bd[h][2], bd[h][3]);
-        }
+    const ulonglong2* rec = reinterpret_cast<const ulonglong2*>(fwd_smem + stage * SST);
+    const ulonglong2* crs = rec + kChunk * kRecFloat4;  // colour mode: this stage's colour records
+#pragma unroll kFwdUnroll
+    for (int i = 0; i < n; i += 2) {
+      const CamRec2 g = cam_load(rec + kRecFloat4 * i);
+      f2 c0 = zero2, c1 = zero2, c2 = zero2;
+      if (COLOR) {
+        const ulonglong2 q0 = crs[i], q1 = crs[i + 1];
+        c0 = as_f2(q0.x);
+        c1 = as_f2(q0.y);
+        c2 = as_f2(q1.x);
       }
-    } else {
-#pragma unroll 2
-      for (int i = 0; i < n; ++i) {
-        const GaussRec g = unpack_rec(rec[kRecFloat4 * i + 0], rec[kRecFloat4 * i + 1], rec[kRecFloat4 * i + 2],
-                                      rec[kRecFloat4 * i + 3]);
-        if (PACKED) {
-          const GaussRec2 g2 = broadcast_rec(g);
-          const float4 col = COLOR ? crs[i] : float4{};
 #pragma unroll
-          for (int q = 0; q < NP; ++q) fwd_pair2<NORMALS, COLOR>(A2[q], g2, K2v, K3v, B1v, tiny, col);
-        } else {
-#pragma unroll
-          for (int r = 0; r < NA; ++r) fwd_pair<NORMALS>(A[r], g, k);
-        }
-      }
+      for (int r = 0; r < RPT; ++r) fwd_pair2<NORMALS, COLOR>(A[r], g, nB1, tiny, c0, c1, c2);
     }
     __syncthreads();  // every thread is done with this stage before it is refilled
     if (tid == 0 && c + 2 < nchunks) {
-      const int n2 = min(kChunk, K - (c + 2) * kChunk);
+      const int n2 = (min(kChunk, K - (c + 2) * kChunk) + 1) & ~1;
       mbar_arrive_expect_tx(&bars[stage], n2 * 16u * (kRecFloat4 + (COLOR ? 1 : 0)));
       if (COLOR)
         bulk_g2s(fwd_smem + stage * SST + kChunk * kRecFloat4, csrc + (c + 2) * kChunk, n2 * 16u, &bars[stage]);
@@ -474,11 +661,11 @@ __global__ void __launch_bounds__(kFwdThreads, COLOR ? 0 : fwd_min_blocks<NORMAL
 #pragma unroll
     for (int r = 0; r < RPT; ++r) {
       if (pix[r] >= P) continue;
-      const RayAcc a = ray_acc_of<PACKED, NA, NP>(A, A2, r);
+      const RaySums a = ray_sums(A[r]);
       float4* q = reinterpret_cast<float4*>(out.part + V.part_off +
                                             8 * (static_cast<long long>(pix[r]) * V.n_gblocks + ks));
       q[0] = make_float4(a.m, a.Sw, a.Swt, a.Sd);
-      q[1] = make_float4(a.N0, a.N1, a.N2, 0.f);
+      q[1] = make_float4(a.N0, a.N1, 0.f, 0.f);
     }
     continue;
   }
@@ -497,21 +684,22 @@ __global__ void __launch_bounds__(kFwdThreads, COLOR ? 0 : fwd_min_blocks<NORMAL
   const float o[3] = {o0, o1, o2};
 #pragma unroll
   for (int r = 0; r < RPT; ++r) {
-    if (pix[r] >= P) continue;
     const long long p = pix[r];
-    const RayAcc a = ray_acc_of<PACKED, NA, NP>(A, A2, r);
+    const bool in = pix[r] < P;
+    const RaySums a = ray_sums(A[r]);
+    const CamRay ray = cam_ray(V, ray_pixel(V, min(pix[r], P - 1)));
+    RayNormal N{0.f, 0.f, 0.f};
+    if (NORMALS) N = ray_normal_checked(V, s, k, a, ray, pix[r], in);
+    if (!in) continue;
     if (COLOR) {
       const float iSw = 1.0f / a.Sw;
-      const RayAcc2& b = A2[r / 2];
-      const bool h = (r & 1) != 0;
       float* col = out.color + 3 * off;
-      col[p] = (h ? hi(b.C0) : lo(b.C0)) * iSw;
-      col[P + p] = (h ? hi(b.C1) : lo(b.C1)) * iSw;
-      col[2 * P + p] = (h ? hi(b.C2) : lo(b.C2)) * iSw;
+      col[p] = a.C0 * iSw;
+      col[P + p] = a.C1 * iSw;
+      col[2 * P + p] = a.C2 * iSw;
     }
-    write_ray_outputs<NORMALS, NFLOW>(V, R, o, Rj, tj, has_t, a, pxy[r], p, out);
+    write_ray_outputs<NORMALS, NFLOW>(V, R, o, Rj, tj, has_t, a, N, ray, p, out);
   }
-  (void)vc;
   }  // item loop
 }
 
@@ -523,16 +711,16 @@ static int fwd_smem_bytes(int maxK, bool color = false) {
 template <bool NORMALS, int NFLOW, int RPT>
 static int fwd_ctas_per_sm_t(int maxK) {
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, forward_kernel<NORMALS, NFLOW, RPT, false>, kFwdThreads,
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, forward_kernel<NORMALS, NFLOW, RPT>, kFwdThreads,
                                                     fwd_smem_bytes(maxK)) != cudaSuccess)
     return 1;
   return n > 0 ? n : 1;
 }
 
-template <bool NORMALS, int NFLOW, int RPT, bool STORE = false, bool COLOR = false, class B>
+template <bool NORMALS, int NFLOW, int RPT, bool COLOR = false, class B>
 static cudaError_t launch_fwd_t(const B& b, const Scene& s, const Consts& c, const float4* records,
                                 const FwdOut& o, int maxK, int* status, int* counter, cudaStream_t st) {
-  auto kern = forward_kernel<NORMALS, NFLOW, RPT, STORE, COLOR, B>;
+  auto kern = forward_kernel<NORMALS, NFLOW, RPT, COLOR, B>;
   const int smem = fwd_smem_bytes(maxK, COLOR);
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -551,10 +739,8 @@ static cudaError_t launch_fwd_t(const B& b, const Scene& s, const Consts& c, con
 template <bool NORMALS, int NFLOW, class B>
 static cudaError_t launch_fwd_r(int rpt, const B& b, const Scene& s, const Consts& c, const float4* records,
                                 const FwdOut& o, int maxK, int* status, int* counter, cudaStream_t st) {
-  if (o.pairs != nullptr)  // stored-intermediate mode: two rays per thread only
-    return launch_fwd_t<NORMALS, NFLOW, 2, true>(b, s, c, records, o, maxK, status, counter, st);
   if (o.color != nullptr)  // colour mode: two rays per thread only
-    return launch_fwd_t<NORMALS, NFLOW, 2, false, true>(b, s, c, records, o, maxK, status, counter, st);
+    return launch_fwd_t<NORMALS, NFLOW, 2, true>(b, s, c, records, o, maxK, status, counter, st);
   switch (rpt) {
     case 1: return launch_fwd_t<NORMALS, NFLOW, 1>(b, s, c, records, o, maxK, status, counter, st);
     case 2: return launch_fwd_t<NORMALS, NFLOW, 2>(b, s, c, records, o, maxK, status, counter, st);
@@ -598,14 +784,15 @@ int forward_merge_rays_per_item() { return kMergeThreads; }
 
 template <bool NORMALS, int NFLOW, class B>
 __global__ void __launch_bounds__(kMergeThreads) fwd_merge_kernel(const __grid_constant__ B batch, Scene s,
-                                                                  FwdOut out) {
+                                                                  Consts c, FwdOut out) {
   pdl_enter();
   int local;
   const int vi = find_item(batch, blockIdx.x, local);
   const DevView& V = batch.v[vi];
   const int P = V.P;
-  const long long p = static_cast<long long>(local) * kMergeThreads + threadIdx.x;
-  if (p >= P) return;
+  const bool in = local * kMergeThreads + static_cast<int>(threadIdx.x) < P;
+  // threads past the end merge a valid ray and store nothing
+  const long long p = min(local * kMergeThreads + static_cast<int>(threadIdx.x), P - 1);
   float R[9], tp[3];
   load_pose(s.poses, V.pose, R, tp);
   const float o[3] = {-fmaf(R[6], tp[2], fmaf(R[3], tp[1], R[0] * tp[0])),
@@ -619,21 +806,12 @@ __global__ void __launch_bounds__(kMergeThreads) fwd_merge_kernel(const __grid_c
     has_t[j] = tg >= 0;
     if (has_t[j]) load_pose(s.poses, tg, Rj[j], tj[j]);
   }
-  float vc[3], v[3], vl[3], pxy[2];
-  pixel_ray_dd(V, R, ray_pixel(V, static_cast<int>(p)), vc, v, vl, pxy);
+  const CamRay ray = cam_ray(V, ray_pixel(V, static_cast<int>(p)));
   const int S = V.S;  // splits of this view
   const float4* q = reinterpret_cast<const float4*>(out.part + V.part_off + 8 * p * S);
   float m = -INFINITY;
   for (int k = 0; k < S; ++k) m = fmaxf(m, q[2 * k].x);
-  RayAcc a;
-  a.v0 = v[0];
-  a.v1 = v[1];
-  a.v2 = v[2];
-  a.vl0 = vl[0];
-  a.vl1 = vl[1];
-  a.vl2 = vl[2];
-  a.m = m;
-  a.Sw = a.Swt = a.Sd = a.N0 = a.N1 = a.N2 = 0.f;
+  RaySums a{m, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   for (int k = 0; k < S; ++k) {
     const float4 q0 = q[2 * k], q1 = q[2 * k + 1];
     const float sc = ex2_approx(q0.x - m);
@@ -643,33 +821,34 @@ __global__ void __launch_bounds__(kMergeThreads) fwd_merge_kernel(const __grid_c
     if (NORMALS) {
       a.N0 = fmaf(sc, q1.x, a.N0);
       a.N1 = fmaf(sc, q1.y, a.N1);
-      a.N2 = fmaf(sc, q1.z, a.N2);
     }
   }
-  write_ray_outputs<NORMALS, NFLOW>(V, R, o, Rj, tj, has_t, a, pxy, p, out);
+  RayNormal N{0.f, 0.f, 0.f};
+  if (NORMALS) N = ray_normal_checked(V, s, c, a, ray, static_cast<int>(p), in);
+  if (in) write_ray_outputs<NORMALS, NFLOW>(V, R, o, Rj, tj, has_t, a, N, ray, p, out);
 }
 
 template <class B>
-static cudaError_t launch_forward_merge_t(const B& b, const Scene& s, bool normals, int n_flow, const FwdOut& o,
+static cudaError_t launch_forward_merge_t(const B& b, const Scene& s, const Consts& c, bool normals, int n_flow, const FwdOut& o,
                                           cudaStream_t st) {
   if (b.n_items <= 0) return cudaSuccess;
   const dim3 grid(b.n_items), block(kMergeThreads);
   if (normals) {
-    if (n_flow == 0) return launch_kernel(fwd_merge_kernel<true, 0, B>, grid, block, 0, st, 1, b, s, o);
-    if (n_flow == 1) return launch_kernel(fwd_merge_kernel<true, 1, B>, grid, block, 0, st, 1, b, s, o);
-    return launch_kernel(fwd_merge_kernel<true, 2, B>, grid, block, 0, st, 1, b, s, o);
+    if (n_flow == 0) return launch_kernel(fwd_merge_kernel<true, 0, B>, grid, block, 0, st, 1, b, s, c, o);
+    if (n_flow == 1) return launch_kernel(fwd_merge_kernel<true, 1, B>, grid, block, 0, st, 1, b, s, c, o);
+    return launch_kernel(fwd_merge_kernel<true, 2, B>, grid, block, 0, st, 1, b, s, c, o);
   }
-  if (n_flow == 0) return launch_kernel(fwd_merge_kernel<false, 0, B>, grid, block, 0, st, 1, b, s, o);
-  if (n_flow == 1) return launch_kernel(fwd_merge_kernel<false, 1, B>, grid, block, 0, st, 1, b, s, o);
-  return launch_kernel(fwd_merge_kernel<false, 2, B>, grid, block, 0, st, 1, b, s, o);
+  if (n_flow == 0) return launch_kernel(fwd_merge_kernel<false, 0, B>, grid, block, 0, st, 1, b, s, c, o);
+  if (n_flow == 1) return launch_kernel(fwd_merge_kernel<false, 1, B>, grid, block, 0, st, 1, b, s, c, o);
+  return launch_kernel(fwd_merge_kernel<false, 2, B>, grid, block, 0, st, 1, b, s, c, o);
 }
-cudaError_t launch_forward_merge(const Batch& b, const Scene& s, bool normals, int n_flow, const FwdOut& o,
-                                 cudaStream_t st) {
-  return launch_forward_merge_t(b, s, normals, n_flow, o, st);
+cudaError_t launch_forward_merge(const Batch& b, const Scene& s, const Consts& c, bool normals, int n_flow,
+                                 const FwdOut& o, cudaStream_t st) {
+  return launch_forward_merge_t(b, s, c, normals, n_flow, o, st);
 }
-cudaError_t launch_forward_merge(const BigBatch& b, const Scene& s, bool normals, int n_flow, const FwdOut& o,
-                                 cudaStream_t st) {
-  return launch_forward_merge_t(b, s, normals, n_flow, o, st);
+cudaError_t launch_forward_merge(const BigBatch& b, const Scene& s, const Consts& c, bool normals, int n_flow,
+                                 const FwdOut& o, cudaStream_t st) {
+  return launch_forward_merge_t(b, s, c, normals, n_flow, o, st);
 }
 
 int forward_ctas_per_sm(bool normals, int n_flow, int rpt, int maxK) {

@@ -458,6 +458,11 @@ cudaError_t launch_prologue(const Batch& b, const Scene& s, const Consts& c, flo
 cudaError_t launch_prologue(const BigBatch& b, const Scene& s, const Consts& c, float4* records, int maxK,
                             int* status_to_clear, int* counter_to_clear, cudaStream_t st,
                             const ZeroJob* zero = nullptr);
+// The camera-plane render's records (fmb_cam.cuh).
+cudaError_t launch_prologue_cam(const Batch& b, const Scene& s, float4* records, int maxK, int* status_to_clear,
+                                int* counter_to_clear, cudaStream_t st, const ZeroJob* zero = nullptr);
+cudaError_t launch_prologue_cam(const BigBatch& b, const Scene& s, float4* records, int maxK, int* status_to_clear,
+                                int* counter_to_clear, cudaStream_t st, const ZeroJob* zero = nullptr);
 // counter: persistent mode's work counter (zeroed before the launch), or null for
 // one CTA per work item.
 struct FwdOut;
@@ -467,13 +472,24 @@ cudaError_t launch_forward(const Batch& b, const Scene& s, const Consts& c, cons
 cudaError_t launch_forward(const BigBatch& b, const Scene& s, const Consts& c, const float4* records, bool normals,
                            int n_flow, int rpt, int maxK, const FwdOut& o, int* status, int* counter,
                            cudaStream_t st);
+// The same in the world-frame form (fmb_world_fwd.cu, fmb_world_bwd.cu).
+cudaError_t launch_forward_world(const Batch& b, const Scene& s, const Consts& c, const float4* records, bool normals,
+                                 int n_flow, int rpt, int maxK, const FwdOut& o, int* status, int* counter,
+                                 cudaStream_t st);
+cudaError_t launch_forward_world(const BigBatch& b, const Scene& s, const Consts& c, const float4* records, bool normals,
+                                 int n_flow, int rpt, int maxK, const FwdOut& o, int* status, int* counter,
+                                 cudaStream_t st);
+cudaError_t launch_forward_merge_world(const Batch& b, const Scene& s, bool normals, int n_flow, const FwdOut& o,
+                                       cudaStream_t st);
+cudaError_t launch_forward_merge_world(const BigBatch& b, const Scene& s, bool normals, int n_flow, const FwdOut& o,
+                                       cudaStream_t st);
 // Gaussian-split forward: the merge of the splits' partial sums (o.part) into the
 // planes; work items of forward_merge_rays_per_item() rays, the split count in DevView::S.
 int forward_merge_rays_per_item();
-cudaError_t launch_forward_merge(const Batch& b, const Scene& s, bool normals, int n_flow, const FwdOut& o,
-                                 cudaStream_t st);
-cudaError_t launch_forward_merge(const BigBatch& b, const Scene& s, bool normals, int n_flow, const FwdOut& o,
-                                 cudaStream_t st);
+cudaError_t launch_forward_merge(const Batch& b, const Scene& s, const Consts& c, bool normals, int n_flow,
+                                 const FwdOut& o, cudaStream_t st);
+cudaError_t launch_forward_merge(const BigBatch& b, const Scene& s, const Consts& c, bool normals, int n_flow,
+                                 const FwdOut& o, cudaStream_t st);
 
 struct FwdOut {
   float* depth;
@@ -518,6 +534,12 @@ cudaError_t launch_backward(const Batch& b, const Scene& s, const Consts& c, con
 cudaError_t launch_backward(const BigBatch& b, const Scene& s, const Consts& c, const float4* records, bool normals,
                             int n_flow, int ray_tile, int threads, const BwdIn& in, const BwdOut& out,
                             int* counter, cudaStream_t st);
+cudaError_t launch_backward_world(const Batch& b, const Scene& s, const Consts& c, const float4* records, bool normals,
+                                  int n_flow, int ray_tile, int threads, const BwdIn& in, const BwdOut& out,
+                                  int* counter, cudaStream_t st);
+cudaError_t launch_backward_world(const BigBatch& b, const Scene& s, const Consts& c, const float4* records, bool normals,
+                                  int n_flow, int ray_tile, int threads, const BwdIn& in, const BwdOut& out,
+                                  int* counter, cudaStream_t st);
 // Resident CTAs per SM of the render kernels for this configuration (persistent
 // grid sizing).
 int forward_ctas_per_sm(bool normals, int n_flow, int rpt, int maxK);
