@@ -20,7 +20,7 @@ BUILD_DIR = os.path.join(PKG, "_build")
 LIB_DIR = os.path.join(PKG, "_lib")
 LIB_PATH = os.path.join(LIB_DIR, "libfmb.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["fmb_forward.cu", "fmb_backward.cu", "fmb_world_fwd.cu", "fmb_world_bwd.cu", "fmb_ac.cu", "fmb_points.cu", "fmb_attrib.cu", "fmb_api.cu",
+SOURCES = ["fmb_forward.cu", "fmb_backward.cu", "fmb_world_fwd.cu", "fmb_world_bwd.cu", "fmb_ac.cu", "fmb_ac_walk.cu", "fmb_points.cu", "fmb_attrib.cu", "fmb_api.cu",
            "fmb_probe.cu", "fmb_adam.cu"]
 # Per-source flags.  The backward's scalar code (the per-ray records, the
 # finalisation) is compiled in fast-math mode: subnormals flush to zero, division
@@ -31,7 +31,8 @@ SOURCES = ["fmb_forward.cu", "fmb_backward.cu", "fmb_world_fwd.cu", "fmb_world_b
 # alpha-compositing unit (orbit forward 1.764 -> 1.715 ms, backward 3.844 -> 3.746
 # ms); the two-parameter forward is slower in this mode and keeps the default.
 EXTRA_FLAGS = {"fmb_backward.cu": ["--use_fast_math"], "fmb_world_bwd.cu": ["--use_fast_math"],
-               "fmb_ac.cu": ["--use_fast_math"]}
+               "fmb_ac.cu": ["--use_fast_math"],
+               "fmb_ac_walk.cu": ["--use_fast_math"]}
 
 
 def nvcc() -> str:

@@ -466,6 +466,10 @@ __global__ void __launch_bounds__(kAcThreads, M >= 8 ? 2 : (TPR ? 4 : 3)) backwa
       float Dref = in.depth[off + p];  // centres the depth sums (any finite value is exact)
       if (!(fabsf(Dref) < 1e30f)) Dref = 0.f;
       const float4* crec = color ? s.crec + V.rec_off : nullptr;
+      // Without normals the first pass leaves (t, delta) where the second writes its
+      // values, so that a pair is evaluated once (orbit adjoint without normals, K = 100:
+      // 1.725 -> 1.589 ms).
+      float2* pv = reinterpret_cast<float2*>(pairv) + rr * 32 * M;
       constexpr int NS = 8;  // sums: w, w (t - Dref), w n (3), w c (3)
       bool ok = K >= 8;
       float Sc = 0.f, tl = -INFINITY, t0 = INFINITY;
@@ -477,6 +481,7 @@ __global__ void __launch_bounds__(kAcThreads, M >= 8 ? 2 : (TPR ? 4 : 3)) backwa
         const int e = orow[i];
         ok = ok && e < K;
         const AcPair q = ac_pair_eval<NORMALS>(srec + kAcRecStride * (e < K ? e : 0), v, vl, k);
+        if (!NORMALS) pv[e < K ? e : 0] = make_float2(q.t, q.dl);
         ok = ok && q.t > tl;  // strictly increasing: a sorted permutation without ties
         if (i == c0) t0 = q.t;
         tl = q.t;
@@ -519,7 +524,6 @@ __global__ void __launch_bounds__(kAcThreads, M >= 8 ? 2 : (TPR ? 4 : 3)) backwa
                                                               Dref + Dc, N, Sd, color, want_pose && use && sub == 0,
                                                               pose_acc);
       if (use) {
-        float2* pv = reinterpret_cast<float2*>(pairv) + rr * 32 * M;
         float S2 = 0.f;
         float run[NS];
 #pragma unroll
@@ -527,7 +531,13 @@ __global__ void __launch_bounds__(kAcThreads, M >= 8 ? 2 : (TPR ? 4 : 3)) backwa
 #pragma unroll 2
         for (int i = c0; i < c1; ++i) {
           const int e = orow[i];
-          const AcPair q = ac_pair_eval<NORMALS>(srec + kAcRecStride * e, v, vl, k);
+          AcPair q;
+          if (NORMALS) {
+            q = ac_pair_eval<NORMALS>(srec + kAcRecStride * e, v, vl, k);
+          } else {
+            const float2 td = pv[e];
+            q = AcPair{td.x, td.y, {0.f, 0.f, 0.f}};
+          }
           const float Tl = ex2_approx(-S2 * kLog2e);
           const float wl = Tl * one_minus_exp_neg(q.dl);
           S2 += q.dl;

@@ -177,7 +177,8 @@ template <bool NORMALS>
 __device__ __forceinline__ AcPair ac_pair_eval(const float4* __restrict__ r, const float v[3], const float vl[3],
                                                const Consts& k) {
   const GaussRec g = unpack_rec(r[0], r[1], r[2], r[3]);
-  const PairGeom G = pair_geom(g.L, g.b, g.mh, g.nbl, v[0], v[1], v[2], vl[0], vl[1], vl[2]);
+  // without normals u enters only q = u.u, which needs no second projection; t is the same
+  const PairGeom G = pair_geom<NORMALS>(g.L, g.b, g.mh, g.nbl, v[0], v[1], v[2], vl[0], vl[1], vl[2]);
   AcPair q;
   q.t = G.t;
   q.dl = ex2_approx(fmaf(G.q, k.K3, g.l2));  // delta (Eq. 4)

@@ -19,6 +19,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "fmb_ac_walk.cuh"
 #include "fmb_internal.cuh"
 
 namespace fmb {
@@ -158,6 +159,7 @@ struct Plan {
   int ray_tile = 480;
   int bwd_threads = 160;
   int ac_run = 1;  // alpha compositing: forward rays per warp
+  int ac_walk = 0;  // alpha compositing: column length of the thread-per-ray forward (0: warp per ray)
   int ksplit = 1;  // two-parameter forward: Gaussian splits per view (1 = unsplit)
   long long fwd_part_floats = 0;  // split forward: per-ray partial sums
   std::vector<fmb::Batch> fmerge;  // split forward: merge launches (one per forward launch)
@@ -310,6 +312,10 @@ void fill_batches(Plan& pl, const fmb_params* p, const long long* offs, int n_vi
       // forward
       fmb::DevView df = d;
       df.n_tiles = static_cast<int>((P + rays_fwd - 1) / rays_fwd);
+      if (pl.ac_walk > 0) {
+        const long long columns = static_cast<long long>(v.W) * ((v.H + pl.ac_walk - 1) / pl.ac_walk);
+        df.n_tiles = static_cast<int>((columns + fmb::ac_walk_threads() - 1) / fmb::ac_walk_threads());
+      }
       {
         // split s renders Gaussians [s GB, min(K, (s + 1) GB)); every split is non-empty
         const int S0 = std::min(pl.ksplit, d.K);
@@ -390,6 +396,9 @@ Plan make_plan(const fmb_params* p, const long long* offs, int n_objects, int n_
     long long total = 0;
     for (int i = 0; i < n_views; ++i) total += view_entries(views[i]);
     pl.ac_run = fmb::ac_fwd_run(total, sms);
+    pl.ac_walk = fmb::ac_walk_run(total, sms);
+    for (int i = 0; i < n_views; ++i)  // the entries of a ray batch are no columns of pixels
+      if (views[i].rays != nullptr) pl.ac_walk = 0;
   }
   const int rays_fwd = ac ? fmb::ac_fwd_rays_per_item(pl.ac_run) : fmb::forward_rays_per_cta(pl.rpt);
   // Gaussian split of the two-parameter forward: when the batch's ray tiles fill
@@ -484,6 +493,15 @@ cudaError_t launch_records(const fmb_params* p, const Plan& pl, const B& b, cons
   if (p->variant == 1 || pl.world)
     return fmb::launch_prologue(b, sc, c, records, maxK, status_to_clear, counter, s, zero);
   return fmb::launch_prologue_cam(b, sc, records, maxK, status_to_clear, counter, s, zero);
+}
+
+cudaError_t launch_ac(const fmb_params* p, const Plan& pl, const fmb::Batch& b, const fmb::Scene& sc,
+                      const fmb::Consts& c, const float4* records, const fmb::FwdOut& fo, int* status, int* counter,
+                      cudaStream_t s) {
+  const bool normals = p->want_normals != 0;
+  return pl.ac_walk > 0
+             ? fmb::launch_forward_ac_walk(b, sc, c, records, normals, p->n_flow, pl.maxK, fo, pl.ac_walk, counter, s)
+             : fmb::launch_forward_ac(b, sc, c, records, normals, p->n_flow, pl.maxK, fo, pl.ac_run, status, counter, s);
 }
 
 fmb_status check_workspace(void* ws, size_t bytes, size_t need) {
@@ -616,8 +634,7 @@ fmb_status fmb_render_forward(const fmb_params* params, int n_objects, const lon
         if constexpr (std::is_same_v<std::decay_t<decltype(b)>, fmb::Batch>) {
           if (params->variant == 1) {  // alpha compositing: 64-view batches only
             fo.pairs = nullptr;
-            e = fmb::launch_forward_ac(b, sc, c, records, params->want_normals != 0, params->n_flow, pl.maxK, fo,
-                                       pl.ac_run, status, counter, s);
+            e = launch_ac(params, pl, b, sc, c, records, fo, status, counter, s);
             if (e != cudaSuccess) return cuda_fail(e, "forward launch");
             continue;
           }
@@ -997,8 +1014,7 @@ extern "C" fmb_status fmb_render_forward_noalloc(const fmb_params* params, int n
       fo.color = color;
       if (params->variant == 1) {
         fo.pairs = nullptr;
-        e = fmb::launch_forward_ac(b, sc, c, records, params->want_normals != 0, params->n_flow, pl.maxK, fo, pl.ac_run,
-                                   status, counter, s);
+        e = launch_ac(params, pl, b, sc, c, records, fo, status, counter, s);
       } else {
         e = pl.world ? fmb::launch_forward_world(b, sc, c, records, params->want_normals != 0, params->n_flow, pl.rpt,
                                                  pl.maxK, fo, status, counter, s)
