@@ -22,7 +22,7 @@ DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "fmb_gb300", "au
 # round trip, where the hardware starts the next CTA of a grid in a freed slot
 # directly and already takes the cost-ordered items most expensive first.
 CANDIDATES = [dict(fwd_rays_per_thread=r, bwd_threads=t, bwd_ray_tile=t * m, use_persistent=0)
-              for r in (2, 4) for t in (128, 160) for m in (2, 3)]
+              for r in (2, 4) for t in (128, 160) for m in (2, 3, 4)]
 
 # Extra candidates for small batches (fewer 256-ray tiles than two waves of the
 # GPU's SMs): short ray tiles and narrow CTAs spread a few thousand rays over more

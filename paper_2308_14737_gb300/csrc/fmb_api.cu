@@ -48,6 +48,12 @@ constexpr int kDefaultRpt = 2;
 // world, 38.1 camera; 50 000-ray minibatch at K = 256, eager calls: 167 and 166 us),
 // while 150 000 rays at K = 100-4096 already gain 1.2-1.35x.
 constexpr long long kWorldRays = 131072;
+// Camera-plane adjoint, atomic mode: the CTAs add their sums into this many slots per
+// view and Gaussian block of the workspace, and the deterministic mode's second stage
+// adds the slots.  Added straight into the gradients, 16 views of 320x240 make 38 400
+// fp32 additions per value, whose rounding (sqrt(n) 2^-25) was most of the gradients'
+// error.
+constexpr int kAccSlots = 8;
 constexpr int kMaxGaussPerCta = 256;
 constexpr long long kMaxK = 1 << 22;
 constexpr int kMaxKAlphaCompositing = 256;
@@ -121,8 +127,10 @@ BwdBlocking bwd_blocking(int K, int T, int min_blocks = 0, bool even_blocks = fa
 
 // Threads per backward CTA: the candidate with the lowest modelled cost over the
 // batch (each view's rays x (K / lane fill + 5 per Gaussian block), as in
-// bwd_blocking).
-int choose_bwd_threads(const fmb_view* views, int n_views, const long long* offs, int min_blocks, bool even_blocks) {
+// bwd_blocking; camera-plane form: 160 threads leave 3 CTAs and 15 warps per SM, 128
+// leave 4 and 16).
+int choose_bwd_threads(const fmb_view* views, int n_views, const long long* offs, int min_blocks, bool even_blocks,
+                       bool world) {
   const int cand[] = {128, 160};
   int best = 160;
   double best_cost = -1.0;
@@ -133,6 +141,7 @@ int choose_bwd_threads(const fmb_view* views, int n_views, const long long* offs
       const BwdBlocking b = bwd_blocking(K, T, min_blocks, even_blocks);
       cost += static_cast<double>(view_entries(views[i])) * (K / bwd_lane_fill(K, T, b.n_gb) + 5.0 * b.n_gb);
     }
+    if (!world && T == 160) cost *= 16.0 / 15.0;
     if (best_cost < 0.0 || cost < best_cost - 1e-9 || (std::fabs(cost - best_cost) <= 1e-9 && T > best)) {
       best_cost = cost;
       best = T;
@@ -260,6 +269,13 @@ bool even_blocks(const fmb_params* p, const Plan& pl) {
   return p->variant == 0 && (!pl.world || p->store_pairs != 0);
 }
 
+// Partial-sum slots per Gaussian block of a view of n_tiles: one per tile in
+// deterministic mode, up to kAccSlots in the camera-plane form's atomic mode.
+bool acc_slots(const fmb_params* p, const Plan& pl) { return p->variant == 0 && !pl.world && !p->deterministic; }
+int part_slots(const fmb_params* p, const Plan& pl, int n_tiles) {
+  return acc_slots(p, pl) ? std::min(kAccSlots, n_tiles) : n_tiles;
+}
+
 long long total_entries(const fmb_view* views, int n_views) {
   long long n = 0;
   for (int i = 0; i < n_views; ++i) n += view_entries(views[i]);
@@ -342,7 +358,7 @@ void fill_batches(Plan& pl, const fmb_params* p, const long long* offs, int n_vi
       db.S = bk.S;
       db.slot_floats = (p->colors ? 13 : 10) * bk.GB + 12 * (1 + n_flow);
       db.part_off = part;
-      part += static_cast<long long>(db.n_tiles) * db.n_gblocks * db.slot_floats;
+      part += static_cast<long long>(part_slots(p, pl, db.n_tiles)) * db.n_gblocks * db.slot_floats;
       ctas_b += static_cast<long long>(db.n_tiles) * db.n_gblocks;
       bb.v[i] = db;
     }
@@ -376,14 +392,23 @@ void fill_batches(Plan& pl, const fmb_params* p, const long long* offs, int n_vi
 Plan make_plan(const fmb_params* p, const long long* offs, int n_objects, int n_views, const fmb_view* views,
                bool allow_big = false) {
   Plan pl;
-  pl.rpt = p->fwd_rays_per_thread > 0 ? p->fwd_rays_per_thread : kDefaultRpt;
-  pl.world = p->variant == 0 && (p->store_pairs || total_entries(views, n_views) <= kWorldRays);
+  const long long entries = total_entries(views, n_views);
+  pl.world = p->variant == 0 && (p->store_pairs || entries <= kWorldRays);
+  // Four rays per thread where that still leaves the camera-plane forward (3 resident
+  // CTAs per SM) four rounds of CTAs: 16 x 320x240 at K = 100 186 against 190 us with
+  // two, 20 x 640x480 at K = 256 without normals 1.44 against 1.52 ms, one 1024x768 view
+  // at K = 4096 4.47 against 4.54 ms; but 1023x767 at K = 333 363 against 358 us.
+  const bool many = p->variant == 0 && !pl.world && !p->colors && entries >= 6144ll * 152;
+  pl.rpt = p->fwd_rays_per_thread > 0 ? p->fwd_rays_per_thread : (many ? 4 : kDefaultRpt);
   pl.bwd_threads = p->bwd_threads > 0
                        ? p->bwd_threads
-                       : choose_bwd_threads(views, n_views, offs, p->bwd_gblocks, even_blocks(p, pl));
+                       : choose_bwd_threads(views, n_views, offs, p->bwd_gblocks, even_blocks(p, pl),
+                                            pl.world || p->variant == 1);
   // default ray tile: three rays per thread in the per-ray phase (balanced, and long
-  // enough to amortise the per-CTA reductions)
-  pl.ray_tile = p->bwd_ray_tile > 0 ? p->bwd_ray_tile : 3 * pl.bwd_threads;
+  // enough to amortise the per-CTA reductions); four in the camera-plane form, whose ray
+  // records are smaller (orbit adjoint 455 -> 449 us, K = 256 without normals 3.03 ->
+  // 2.98 ms for 20 views, one view at K = 4096 10.17 -> 10.20 ms)
+  pl.ray_tile = p->bwd_ray_tile > 0 ? p->bwd_ray_tile : (pl.world ? 3 : 4) * pl.bwd_threads;
   pl.n_gauss = offs[n_objects];
   const bool ac = p->variant == 1;
   int dev = 0, sms = 0;
@@ -441,7 +466,7 @@ Plan make_plan(const fmb_params* p, const long long* offs, int n_objects, int n_
 }
 
 // Workspace: header (status word, work counters) | records | colour records (if
-// colors) | deterministic partials (if deterministic) | per-pair t, e2, delta
+// colors) | partial sums (if deterministic, or in the camera-plane form) | per-pair t, e2, delta
 // arrays (if store_pairs).
 size_t crec_offset(const Plan& pl) {
   return kHeaderBytes + align256(static_cast<size_t>(pl.n_records) * 16 * fmb::kRecFloat4);
@@ -451,7 +476,7 @@ size_t partials_offset(const fmb_params* p, const Plan& pl) {
 }
 size_t pairs_offset(const fmb_params* p, const Plan& pl) {
   size_t bytes = partials_offset(p, pl);
-  if (p->deterministic) bytes += align256(static_cast<size_t>(pl.part_floats) * sizeof(float));
+  if (p->deterministic || acc_slots(p, pl)) bytes += align256(static_cast<size_t>(pl.part_floats) * sizeof(float));
   return bytes;
 }
 
@@ -559,8 +584,8 @@ int fmb_launch_count(const fmb_params* params, int n_objects, const long long* h
                                               : (pl.big ? pl.bwd_big.size() : pl.bwd.size()));
     if (pass == 0) return nb * (2 + (params->variant == 0 && pl.ksplit > 1 ? 1 : 0));  // prologue, forward, merge
     if (nb == 0) return 1;  // the zeroing launch
-    // prologue and backward per batch; deterministic mode adds the Gaussian (and pose) reductions
-    return nb * (2 + (params->deterministic ? 1 + (want_pose ? 1 : 0) : 0));
+    // prologue and backward per batch; deterministic mode (and the camera-plane form) adds the Gaussian (and pose) reductions
+    return nb * (2 + (params->deterministic || acc_slots(params, pl) ? 1 + (want_pose ? 1 : 0) : 0));
   } catch (const std::exception& e) {
     fail(FMB_ERR_INVALID_ARG, e.what());
     return -1;
@@ -691,7 +716,8 @@ fmb_status fmb_render_backward(const fmb_params* params, int n_objects, const lo
     char* base = static_cast<char*>(workspace);
     float4* records = reinterpret_cast<float4*>(base + kHeaderBytes);
     float* partials = nullptr;
-    if (params->deterministic) partials = reinterpret_cast<float*>(base + partials_offset(params, pl));
+    const bool acc = acc_slots(params, pl);
+    if (params->deterministic || acc) partials = reinterpret_cast<float*>(base + partials_offset(params, pl));
     fmb::Scene sc{means, chol, weights, poses};
     if (params->colors) {
       sc.colors = colors;
@@ -704,6 +730,7 @@ fmb_status fmb_render_backward(const fmb_params* params, int n_objects, const lo
     fmb::BwdIn in{depth,   normals ? normal : nullptr, saved, g_depth, g_alpha, normals ? g_normal : nullptr,
                   params->n_flow > 0 ? g_flow : nullptr, pairs, pl.pair_stride};
     fmb::BwdOut out{grad_means, grad_chol, grad_weights, grad_poses, partials};
+    out.slots = acc ? kAccSlots : 0;
     if (params->colors) {
       in.color = color;
       in.g_color = g_color;
@@ -724,6 +751,8 @@ fmb_status fmb_render_backward(const fmb_params* params, int n_objects, const lo
     zj.n[4] = grad_poses ? 12ll * n_poses : 0;
     zj.ptr[5] = params->colors ? grad_colors : nullptr;
     zj.n[5] = params->colors ? 3 * pl.n_gauss : 0;
+    zj.ptr[6] = acc ? partials : nullptr;
+    zj.n[6] = acc ? pl.part_floats : 0;
     cudaError_t e = cudaSuccess;
     int* counter = params->use_persistent ? reinterpret_cast<int*>(base + kBwdCounterOffset) : nullptr;
     bool first = true;  // the first batch's prologue clears the outputs and the status word

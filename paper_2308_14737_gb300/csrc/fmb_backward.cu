@@ -44,14 +44,15 @@
 namespace fmb {
 
 constexpr int kBwdMaxThreads = 160;
-#ifndef FMB_BWD_UNROLL
-#define FMB_BWD_UNROLL 2  // pair-loop unrolling (independent rays the scheduler can interleave)
-#endif
-#ifndef FMB_BWD_MIN_BLOCKS
-#define FMB_BWD_MIN_BLOCKS 3
-#endif
-constexpr int kBwdMinBlocks = FMB_BWD_MIN_BLOCKS;  // resident CTAs per SM the register budget targets
-constexpr int kBwdUnroll = FMB_BWD_UNROLL;
+// Resident CTAs per SM the register budget targets (128 registers; with 2, the orbit 498
+// against 467 us, 20 views 640x480 at K = 256 3.12 against 3.02 ms).
+constexpr int kBwdMinBlocks = 3;
+// Pair-loop unrolling: independent rays the scheduler can interleave (orbit 449 / 459 /
+// 454 us with 3 / 2 / 1, without normals 2.98 / 2.97 / 2.96 ms).
+template <bool NORMALS>
+constexpr int bwd_unroll() {
+  return NORMALS ? 3 : 1;
+}
 
 // Per-thread gradient sums of the thread's two Gaussians (one per lane).  y, abar,
 // B00 .. are scaled and in pixels as the records are (fmb_cam.cuh).
@@ -353,8 +354,7 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
     for (int r = r_lo + tid; r < r_hi; r += T) {
       const int p = pix0 + r;
       const CamRay ray = cam_ray(V, ray_pixel(V, p));
-      const float il = 1.0f / ray.len;
-      const float vc[3] = {ray.x * il, ray.y * il, il};
+      const float vc[3] = {ray.x * ray.ilen, ray.y * ray.ilen, ray.ilen};
       float v[3];
 #pragma unroll
       for (int c = 0; c < 3; ++c) v[c] = fmaf(R[6 + c], vc[2], fmaf(R[3 + c], vc[1], R[c] * vc[0]));
@@ -448,7 +448,8 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
         }
       }
       const float KA = kTwoLn2 * gA * expf(-Sd);
-      const float Dz = Dbar * ray.len, nD = -__fdiv_rn(D, ray.len);
+      const float Dq = __fmul_rn(D, ray.ilen);  // D / |c|, corrected by its remainder
+      const float Dz = Dbar * ray.len, nD = -__fmaf_rn(__fmaf_rn(-Dq, ray.len, D), ray.ilen, Dq);
       constexpr int NR = ray_rec2<NORMALS, COLOR>();
       const float K2 = __fmul_rn(k.K2, ray.len), b2 = k.b2e * ray.len;
       float4 rec[NR];
@@ -506,7 +507,7 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
     const CamRec2 gr = cam_load(reinterpret_cast<const ulonglong2*>(records + kRecFloat4 * rec0));
     const f2 nB1 = dup(-k.beta1), nB1s = dup(-kTwoLn2 * k.beta1), tiny = dup(-1e-30f);
     const ulonglong2* rays = reinterpret_cast<const ulonglong2*>(bsm);
-    constexpr int NR = ray_rec2<NORMALS, COLOR>();
+    constexpr int NR = ray_rec2<NORMALS, COLOR>(), kUnroll = bwd_unroll<NORMALS>();
     f2 c0 = dup(0.f), c1 = c0, c2 = c0;  // the two Gaussians' colours, one per lane
     if (COLOR) {
       const ulonglong2* cr = reinterpret_cast<const ulonglong2*>(s.crec + rec0);
@@ -514,7 +515,7 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
       c1 = as_f2(cr[0].y);
       c2 = as_f2(cr[1].x);
     }
-#pragma unroll kBwdUnroll
+#pragma unroll kUnroll
     for (int r = sg; r < nr; r += S)
       bwd_pair2<NORMALS, COLOR, POSE>(A, gr, rays + NR * r, nB1, nB1s, tiny, c0, c1, c2);
   }
@@ -531,8 +532,10 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
   __syncthreads();
   float* slot = nullptr;
   if (out.partials) {
-    slot = out.partials + V.part_off + static_cast<long long>(tile * V.n_gblocks + gb) * V.slot_floats;
+    const int t = out.slots > 0 ? tile % out.slots : tile;
+    slot = out.partials + V.part_off + static_cast<long long>(t * V.n_gblocks + gb) * V.slot_floats;
   }
+  const bool accumulate = out.slots > 0;
   float pose_g[12];
 #pragma unroll
   for (int i = 0; i < 12; ++i) pose_g[i] = 0.f;
@@ -570,13 +573,13 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
       }
     } else {
       float* d = slot + NC * gi;
-      d[0] = gm[0]; d[1] = gm[1]; d[2] = gm[2];
+      const float v[13] = {gm[0], gm[1], gm[2], gL[0], gL[1], gL[2], gL[3], gL[4], gL[5], glam, gcol[0], gcol[1], gcol[2]};
+      if (!accumulate) {
 #pragma unroll
-      for (int i = 0; i < 6; ++i) d[3 + i] = gL[i];
-      d[9] = glam;
-      if (COLOR) {
+        for (int i = 0; i < NC; ++i) d[i] = v[i];
+      } else if (g < V.K) {
 #pragma unroll
-        for (int k3 = 0; k3 < 3; ++k3) d[10 + k3] = gcol[k3];
+        for (int i = 0; i < NC; ++i) atomicAdd(d + i, v[i]);
       }
     }
   }
@@ -593,7 +596,9 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
       float x = 0.f;
       const int nw = (T + 31) / 32;
       for (int w = 0; w < nw; ++w) x += pose_ray[w][tid] + (tid < 12 ? pose_gau[w][tid] : 0.f);
-      if (slot != nullptr) {
+      if (slot != nullptr && accumulate) {
+        atomicAdd(slot + NC * GB + tid, x);
+      } else if (slot != nullptr) {
         slot[NC * GB + tid] = x;
       } else {
         const int j = tid / 12 - 1;
@@ -748,7 +753,7 @@ __device__ __forceinline__ float warp_sum_fixed(float x) {
 template <class B>
 __global__ void reduce_gauss_kernel(const __grid_constant__ B batch, const float* __restrict__ partials,
                                     float* gmeans, float* gchol, float* gweights, float* gcolors, long long n_gauss,
-                                    int nc) {
+                                    int nc, int slots) {
   pdl_enter();
   const long long w = (blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -763,7 +768,8 @@ __global__ void reduce_gauss_kernel(const __grid_constant__ B batch, const float
     hit = true;
     const int gi = static_cast<int>(g - V.gauss_off);
     const int gbk = gi / V.GB, gl = gi - gbk * V.GB;
-    for (int t = lane; t < V.n_tiles; t += 32)
+    const int n = slots > 0 ? min(slots, V.n_tiles) : V.n_tiles;
+    for (int t = lane; t < n; t += 32)
       acc += partials[V.part_off + static_cast<long long>(t * V.n_gblocks + gbk) * V.slot_floats + nc * gl + comp];
   }
   acc = warp_sum_fixed(acc);
@@ -781,7 +787,7 @@ __global__ void reduce_gauss_kernel(const __grid_constant__ B batch, const float
 // Pose gradients: warp w handles (pose p, component comp), w = p * 12 + comp.
 template <class B>
 __global__ void reduce_pose_kernel(const __grid_constant__ B batch, const float* __restrict__ partials,
-                                   float* gposes, int n_poses, int n_flow, int nc) {
+                                   float* gposes, int n_poses, int n_flow, int nc, int slots) {
   pdl_enter();
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -794,7 +800,7 @@ __global__ void reduce_pose_kernel(const __grid_constant__ B batch, const float*
       const int pidx = j < 0 ? V.pose : (j == 0 ? V.tgt0 : V.tgt1);
       if (pidx != p) continue;
       const int part = 12 * (j + 1) + comp;
-      const int nslots = V.n_tiles * V.n_gblocks;
+      const int nslots = (slots > 0 ? min(slots, V.n_tiles) : V.n_tiles) * V.n_gblocks;
       for (int sl = lane; sl < nslots; sl += 32)
         acc += partials[V.part_off + static_cast<long long>(sl) * V.slot_floats + nc * V.GB + part];
     }
@@ -811,10 +817,10 @@ static cudaError_t launch_backward_reduce_t(const B& b, int n_flow, long long n_
   const dim3 grid(static_cast<unsigned>((warps * 32 + 255) / 256));
   const float* partials = out.partials;
   cudaError_t e = launch_kernel(reduce_gauss_kernel<B>, grid, dim3(256), 0, st, 1, b, partials, out.gmeans,
-                                out.gchol, out.gweights, out.gcolors, n_gauss, nc);
+                                out.gchol, out.gweights, out.gcolors, n_gauss, nc, out.slots);
   if (e != cudaSuccess || out.gposes == nullptr) return e;
   return launch_kernel(reduce_pose_kernel<B>, dim3((n_poses * 12 * 32 + 255) / 256), dim3(256), 0, st, 1, b,
-                       partials, out.gposes, n_poses, n_flow, nc);
+                       partials, out.gposes, n_poses, n_flow, nc, out.slots);
 }
 cudaError_t launch_backward_reduce(const Batch& b, int n_flow, long long n_gauss, int n_poses, const BwdOut& out,
                                    cudaStream_t st) {

@@ -297,64 +297,94 @@ struct RayAcc2 {
 // component is -(x g_0 + y g_1) and |g|^2 a quadratic form of the first two, written
 // as (r00 h0 + r01 h1)^2 + (r11 h1)^2 for h = (g_0 / fx, g_1 / fy).
 __device__ __forceinline__ void ray_metric(const DevView& V, const CamRay& r, float& r00, float& r01, float& r11) {
-  const float s = sqrtf(fmaf(r.x, r.x, 1.0f));
-  r00 = V.fx * s;
-  r01 = V.fy * (r.x * r.y / s);
-  r11 = V.fy * (r.len / s);
+  const float s = fmaf(r.x, r.x, 1.0f), is = rsqrt_nr(s);
+  r00 = V.fx * s * is;
+  r01 = V.fy * (r.x * r.y * is);
+  r11 = V.fy * (r.len * is);
+}
+
+// What a pair leaves for the sums once the shift is settled: d, the log2 weight above
+// the shift, t and u.
+struct FwdPair2 {
+  f2 d, t, nx, u0, u1;
+};
+template <bool NORMALS, bool COLOR>
+__device__ __forceinline__ FwdPair2 fwd_pair2(RayAcc2<NORMALS, COLOR>& A, const CamRec2& g, f2 nB1) {
+  const CamGeom2 G = cam_geom2(g, A.X, A.Y);
+  A.Sd = add2(A.Sd, pk(ex2_approx(-lo(G.nx)), ex2_approx(-hi(G.nx))));
+  return FwdPair2{fma2(G.t, A.K2, fma2(G.nx, nB1, A.nm)), G.t, G.nx, G.u0, G.u1};
+}
+
+// Raises the shift of the lane(s) whose exponent it no longer bounds.
+template <bool NORMALS, bool COLOR>
+__device__ __forceinline__ void fwd_raise2(RayAcc2<NORMALS, COLOR>& A, FwdPair2& q, f2 nB1) {
+  const f2 e2 = fma2(q.nx, nB1, mul2(q.t, A.K2));
+  float dl = lo(q.d), dh = hi(q.d), sl = 1.f, sh = 1.f, ml = lo(A.nm), mh = hi(A.nm);
+  if (dl > kLazyShift) {
+    sl = ex2_approx(-(lo(e2) + ml));
+    ml = -lo(e2);
+    dl = 0.f;
+  }
+  if (dh > kLazyShift) {
+    sh = ex2_approx(-(hi(e2) + mh));
+    mh = -hi(e2);
+    dh = 0.f;
+  }
+  const f2 sc = pk(sl, sh);
+  A.Sw = mul2(A.Sw, sc);
+  A.Swt = mul2(A.Swt, sc);
+  if (NORMALS) {
+    A.N0 = mul2(A.N0, sc);
+    A.N1 = mul2(A.N1, sc);
+  }
+  if (COLOR) {
+    A.C0 = mul2(A.C0, sc);
+    A.C1 = mul2(A.C1, sc);
+    A.C2 = mul2(A.C2, sc);
+  }
+  A.nm = pk(ml, mh);
+  q.d = pk(dl, dh);
 }
 
 template <bool NORMALS, bool COLOR>
-__device__ __forceinline__ void fwd_pair2(RayAcc2<NORMALS, COLOR>& A, const CamRec2& g, f2 nB1, f2 tiny, f2 c0,
-                                              f2 c1, f2 c2) {
-  const CamGeom2 G = cam_geom2(g, A.X, A.Y);
-  const f2 delta = pk(ex2_approx(-lo(G.nx)), ex2_approx(-hi(G.nx)));
-  A.Sd = add2(A.Sd, delta);
-  f2 d = fma2(G.t, A.K2, fma2(G.nx, nB1, A.nm));  // log2 weight above the shift
-  if (fmaxf(lo(d), hi(d)) > kLazyShift) {  // rare: raise the shift of the lane(s) it no longer bounds
-    const f2 e2 = fma2(G.nx, nB1, mul2(G.t, A.K2));
-    float dl = lo(d), dh = hi(d), sl = 1.f, sh = 1.f, ml = lo(A.nm), mh = hi(A.nm);
-    if (dl > kLazyShift) {
-      sl = ex2_approx(-(lo(e2) + ml));
-      ml = -lo(e2);
-      dl = 0.f;
-    }
-    if (dh > kLazyShift) {
-      sh = ex2_approx(-(hi(e2) + mh));
-      mh = -hi(e2);
-      dh = 0.f;
-    }
-    const f2 sc = pk(sl, sh);
-    A.Sw = mul2(A.Sw, sc);
-    A.Swt = mul2(A.Swt, sc);
-    if (NORMALS) {
-      A.N0 = mul2(A.N0, sc);
-      A.N1 = mul2(A.N1, sc);
-    }
-    if (COLOR) {
-      A.C0 = mul2(A.C0, sc);
-      A.C1 = mul2(A.C1, sc);
-      A.C2 = mul2(A.C2, sc);
-    }
-    A.nm = pk(ml, mh);
-    d = pk(dl, dh);
-  }
-  const f2 w = ex2_2(d);
+__device__ __forceinline__ void fwd_sum2(RayAcc2<NORMALS, COLOR>& A, const CamRec2& g, const FwdPair2& q, f2 tiny, f2 c0,
+                                         f2 c1, f2 c2) {
+  const f2 w = ex2_2(q.d);
   A.Sw = add2(A.Sw, w);
-  A.Swt = fma2(w, G.t, A.Swt);
+  A.Swt = fma2(w, q.t, A.Swt);
   if (COLOR) {
     A.C0 = fma2(w, c0, A.C0);
     A.C1 = fma2(w, c1, A.C1);
     A.C2 = fma2(w, c2, A.C2);
   }
   if (NORMALS) {
-    const f2 h0 = mul2(g.B00, G.u0);
-    const f2 h1 = fma2(g.B11, G.u1, mul2(g.B10, G.u0));
+    const f2 h0 = mul2(g.B00, q.u0);
+    const f2 h1 = fma2(g.B11, q.u1, mul2(g.B10, q.u0));
     const f2 p0 = fma2(A.r01, h1, mul2(A.r00, h0));
     const f2 p1 = mul2(A.r11, h1);
     const f2 ws = mul2(w, rsqrt_2(fma2(p0, p0, fma2(p1, p1, tiny))));
     A.N0 = fma2(ws, h0, A.N0);
     A.N1 = fma2(ws, h1, A.N1);
   }
+}
+
+// One record against the thread's rays, with one check of the shifts for all of them (a
+// check per ray cost 6 to 9 % of the kernel).
+template <int RPT, bool NORMALS, bool COLOR>
+__device__ __forceinline__ void fwd_record2(RayAcc2<NORMALS, COLOR> (&A)[RPT], const CamRec2& g, f2 nB1, f2 tiny, f2 c0,
+                                            f2 c1, f2 c2) {
+  FwdPair2 q[RPT];
+#pragma unroll
+  for (int r = 0; r < RPT; ++r) q[r] = fwd_pair2<NORMALS, COLOR>(A[r], g, nB1);
+  float top = fmaxf(lo(q[0].d), hi(q[0].d));
+#pragma unroll
+  for (int r = 1; r < RPT; ++r) top = fmaxf(top, fmaxf(lo(q[r].d), hi(q[r].d)));
+  if (top > kLazyShift) {  // rare
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) fwd_raise2<NORMALS, COLOR>(A[r], q[r], nB1);
+  }
+#pragma unroll
+  for (int r = 0; r < RPT; ++r) fwd_sum2<NORMALS, COLOR>(A[r], g, q[r], tiny, c0, c1, c2);
 }
 
 // A ray's sums with the two lanes brought to one shift and added.
@@ -383,7 +413,7 @@ struct RayNormal {
   float n0, n1, n2;
 };
 __device__ __forceinline__ RayNormal ray_normal(const DevView& V, const RaySums& a, const CamRay& ray) {
-  const float iSw = 1.0f / a.Sw;
+  const float iSw = rcp_nr(a.Sw);
   const float N0 = V.fx * a.N0 * iSw, N1 = V.fy * a.N1 * iSw;
   return RayNormal{N0, N1, -fmaf(ray.x, N0, ray.y * N1)};
 }
@@ -493,7 +523,7 @@ __device__ __forceinline__ void write_ray_outputs(const DevView& V, const float 
                                                   long long p, const FwdOut& out) {
   const int P = V.P;
   const long long off = V.pix_off;
-  const float iSw = 1.0f / a.Sw;
+  const float iSw = rcp_nr(a.Sw);  // Sw >= 1 / 2: the shift is one of the exponents
   const float Dz = a.Swt * iSw;
   out.depth[off + p] = Dz * ray.len;
   out.alpha[off + p] = -expm1f(-a.Sd);
@@ -501,8 +531,9 @@ __device__ __forceinline__ void write_ray_outputs(const DevView& V, const float 
   sv[p] = a.m + log2f(a.Sw);
   sv[P + p] = a.Sd;
   if (NORMALS) {
-    const float Nn = sqrtf(fmaf(N.n0, N.n0, fmaf(N.n1, N.n1, N.n2 * N.n2)));
-    const float iN = Nn > 0.f ? 1.0f / Nn : 0.f;
+    const float NN = fmaf(N.n0, N.n0, fmaf(N.n1, N.n1, N.n2 * N.n2));
+    const float iN = NN > 1e-37f ? rsqrt_nr(NN) : (NN == NN ? 0.f : NN);
+    const float Nn = NN * iN;
     float* nrm = out.normal + 3 * off;
     nrm[p] = N.n0 * iN;
     nrm[P + p] = N.n1 * iN;
@@ -523,7 +554,7 @@ __device__ __forceinline__ void write_ray_outputs(const DevView& V, const float 
         const float X0 = fmaf(Rj[j][2], pt[2], fmaf(Rj[j][1], pt[1], fmaf(Rj[j][0], pt[0], tj[j][0])));
         const float X1 = fmaf(Rj[j][5], pt[2], fmaf(Rj[j][4], pt[1], fmaf(Rj[j][3], pt[0], tj[j][1])));
         const float X2 = fmaf(Rj[j][8], pt[2], fmaf(Rj[j][7], pt[1], fmaf(Rj[j][6], pt[0], tj[j][2])));
-        const float iz = 1.0f / X2;
+        const float iz = rcp_nr(X2);
         fu = fmaf(V.fx * X0, iz, V.cx) - ray.px;
         fv = fmaf(V.fy * X1, iz, V.cy) - ray.py;
       }
@@ -639,8 +670,7 @@ __global__ void __launch_bounds__(kFwdThreads)
         c1 = as_f2(q0.y);
         c2 = as_f2(q1.x);
       }
-#pragma unroll
-      for (int r = 0; r < RPT; ++r) fwd_pair2<NORMALS, COLOR>(A[r], g, nB1, tiny, c0, c1, c2);
+      fwd_record2<RPT, NORMALS, COLOR>(A, g, nB1, tiny, c0, c1, c2);
     }
     __syncthreads();  // every thread is done with this stage before it is refilled
     if (tid == 0 && c + 2 < nchunks) {
@@ -687,12 +717,12 @@ __global__ void __launch_bounds__(kFwdThreads)
     const long long p = pix[r];
     const bool in = pix[r] < P;
     const RaySums a = ray_sums(A[r]);
-    const CamRay ray = cam_ray(V, ray_pixel(V, min(pix[r], P - 1)));
+    const CamRay ray = cam_ray_at(V, lo(A[r].X), lo(A[r].Y));
     RayNormal N{0.f, 0.f, 0.f};
     if (NORMALS) N = ray_normal_checked(V, s, k, a, ray, pix[r], in);
     if (!in) continue;
     if (COLOR) {
-      const float iSw = 1.0f / a.Sw;
+      const float iSw = rcp_nr(a.Sw);
       float* col = out.color + 3 * off;
       col[p] = a.C0 * iSw;
       col[P + p] = a.C1 * iSw;

@@ -511,8 +511,10 @@ struct BwdOut {
   float* gchol;
   float* gweights;
   float* gposes;  // may be null
-  float* partials;  // deterministic mode: workspace region, else null
+  float* partials;  // workspace region of partial sums (see slots), or null: add into the outputs
   float* gcolors = nullptr;  // colour mode: [G][3]
+  int slots = 0;             // partials: 0 = one slot per tile (deterministic mode), else that many per
+                             // view and block, into which the tiles accumulate (tile mod slots)
 };
 struct BwdIn {
   const float* depth;
