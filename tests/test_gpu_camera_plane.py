@@ -119,6 +119,35 @@ def test_both_forms_agree(K, normals, rays, opts):
         assert (grads[k].double() - t).abs().max() <= 3e-5 * t.abs().max(), k
 
 
+@pytest.mark.parametrize("K,normals,colors", [(1, 1, 0), (75, 0, 0), (300, 1, 0), (33, 0, 1)])
+def test_gradient_slots_around_their_count(K, normals, colors):
+    """Gradients summed through the slots (views of 1, 2, 3, 7, 8, 9 and 281 tiles of 256
+    rays) against the deterministic mode's one slot per tile: the same
+    terms in another order, to 3e-5 of the largest entry as above."""
+    s = _scene(K, outside=False)
+    base = dict(s.views[0])
+    for n in (1, 2, 3, 7, 8, 9):
+        s.views.append(dict(base, W=16, H=16 * n, fx=30.0, fy=28.0, cx=8.25, cy=8.0 * n, pix_offset=s.n_pixels))
+    assert s.n_pixels > WORLD_RAYS
+    x = dev_scene(s)
+    col = torch.rand(K, 3, device="cuda") if colors else None
+    torch.manual_seed(K)
+    P = s.n_pixels
+    got = []
+    for det in (0, 1):
+        r = fmb.Renderer(s.obj_offsets, s.views, len(s.poses), fmb.default_params(
+            n_flow=1, want_normals=normals, colors=colors, deterministic=det, bwd_ray_tile=256))
+        out = r.forward(*x, colors=col)
+        if det == 0:
+            on = (out["alpha"] >= 1e-2).float()
+            u = [torch.randn(P, device="cuda") * on, torch.randn(P, device="cuda") * on,
+                 torch.zeros(3 * P, device="cuda"), torch.zeros(2 * P, device="cuda")]
+            gc = torch.zeros(3 * P, device="cuda") if colors else None
+        got.append(r.backward(*x, *u, colors=col, g_color=gc))
+    for k, t in got[1].items():
+        assert (got[0][k].double() - t.double()).abs().max() <= 3e-5 * t.abs().max(), k
+
+
 def test_normals_that_cancel():
     """Two equal Gaussians side by side: their normals oppose each other between them, so
     |N| passes through 0 there.  N carries at most 5e-6 (the weights' 1e-5, Sec. 7's
