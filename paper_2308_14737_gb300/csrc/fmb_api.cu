@@ -6,7 +6,7 @@
 //                       backward work counter at 128
 //   [256, 256 + 64 R)   R per-(view, Gaussian) records, R = sum over views of K, each
 //                       view's K rounded up to an even count
-//   [.., ..)            backward partials (deterministic mode only)
+//   [.., ..)            backward partials (deterministic mode and the camera-plane form)
 #include <algorithm>
 #include <cmath>
 #include <cstddef>
@@ -48,12 +48,6 @@ constexpr int kDefaultRpt = 2;
 // world, 38.1 camera; 50 000-ray minibatch at K = 256, eager calls: 167 and 166 us),
 // while 150 000 rays at K = 100-4096 already gain 1.2-1.35x.
 constexpr long long kWorldRays = 131072;
-// Camera-plane adjoint, atomic mode: the CTAs add their sums into this many slots per
-// view and Gaussian block of the workspace, and the deterministic mode's second stage
-// adds the slots.  Added straight into the gradients, 16 views of 320x240 make 38 400
-// fp32 additions per value, whose rounding (sqrt(n) 2^-25) was most of the gradients'
-// error.
-constexpr int kAccSlots = 8;
 constexpr int kMaxGaussPerCta = 256;
 constexpr long long kMaxK = 1 << 22;
 constexpr int kMaxKAlphaCompositing = 256;
@@ -270,10 +264,10 @@ bool even_blocks(const fmb_params* p, const Plan& pl) {
 }
 
 // Partial-sum slots per Gaussian block of a view of n_tiles: one per tile in
-// deterministic mode, up to kAccSlots in the camera-plane form's atomic mode.
+// deterministic mode, up to fmb::kAccSlots in the camera-plane form's atomic mode.
 bool acc_slots(const fmb_params* p, const Plan& pl) { return p->variant == 0 && !pl.world && !p->deterministic; }
 int part_slots(const fmb_params* p, const Plan& pl, int n_tiles) {
-  return acc_slots(p, pl) ? std::min(kAccSlots, n_tiles) : n_tiles;
+  return acc_slots(p, pl) ? std::min(fmb::kAccSlots, n_tiles) : n_tiles;
 }
 
 long long total_entries(const fmb_view* views, int n_views) {
@@ -730,7 +724,7 @@ fmb_status fmb_render_backward(const fmb_params* params, int n_objects, const lo
     fmb::BwdIn in{depth,   normals ? normal : nullptr, saved, g_depth, g_alpha, normals ? g_normal : nullptr,
                   params->n_flow > 0 ? g_flow : nullptr, pairs, pl.pair_stride};
     fmb::BwdOut out{grad_means, grad_chol, grad_weights, grad_poses, partials};
-    out.slots = acc ? kAccSlots : 0;
+    out.slots = acc ? fmb::kAccSlots : 0;
     if (params->colors) {
       in.color = color;
       in.g_color = g_color;
