@@ -297,6 +297,7 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
   __shared__ float pose_gau[kBwdMaxThreads / 32][12];   // per-warp sums of the per-Gaussian pose terms
   __shared__ float view_inv[9];                         // R^-1 of the view's pose
   __shared__ int s_item;
+  if (CL == 2) cluster_arrive();  // this CTA runs: its shared memory may be written by its peer
 
   for (int round = 0;; ++round) {
   const int item = next_item(counter, round, &s_item);
@@ -351,6 +352,7 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
       has_t[j] = tg >= 0 && in.g_flow != nullptr;
       if (has_t[j]) load_pose(s.poses, tg, Rj[j], tj[j]);
     }
+    if (CL == 2) cluster_wait();  // the peer runs: its shared memory may be written (clusters take one item)
     for (int r = r_lo + tid; r < r_hi; r += T) {
       const int p = pix0 + r;
       const CamRay ray = cam_ray(V, ray_pixel(V, p));

@@ -144,14 +144,17 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 // cluster; a 16-byte store to the same shared-memory offset of CTA `rank` of the
 // cluster (distributed shared memory); and a barrier of all threads of the cluster
 // (arrive with release, wait with acquire), after which such stores are visible
-// to every CTA of the cluster.
+// to every CTA of the cluster.  A CTA's shared memory may only be accessed once that
+// CTA runs, so a kernel arrives at its start and waits before its first such store.
 __device__ __forceinline__ uint32_t cluster_ctarank() { return __clusterRelativeBlockRank(); }
 __device__ __forceinline__ void st_cluster_f4(float4* local, int rank, float4 v) {
   *static_cast<float4*>(__cluster_map_shared_rank(local, static_cast<unsigned>(rank))) = v;
 }
+__device__ __forceinline__ void cluster_arrive() { __cluster_barrier_arrive(); }
+__device__ __forceinline__ void cluster_wait() { __cluster_barrier_wait(); }
 __device__ __forceinline__ void cluster_sync() {
-  __cluster_barrier_arrive();
-  __cluster_barrier_wait();
+  cluster_arrive();
+  cluster_wait();
 }
 __device__ __forceinline__ unsigned long long global_timer_ns() {
   unsigned long long t;
