@@ -620,8 +620,9 @@ static int bwd_smem_bytes(int ray_tile, int threads) {
 
 template <bool NORMALS, int NFLOW, bool COLOR = false, bool POSE = true, int CL = 1, class B = Batch>
 static cudaError_t prepare_bwd_t(int smem) {
-  // Dynamic plus static shared memory above the 48 KB default needs the opt-in.
-  if (smem + static_cast<int>(sizeof(float) * (kBwdMaxThreads / 32) * 48) > 48 * 1024)
+  // Dynamic plus static shared memory above the 48 KB default needs the opt-in; the static
+  // part is about 1 KB.
+  if (smem > 46 * 1024)
     return cudaFuncSetAttribute(backward_kernel<NORMALS, NFLOW, COLOR, POSE, CL, B>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   return cudaSuccess;

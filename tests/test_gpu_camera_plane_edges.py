@@ -1,0 +1,62 @@
+"""The camera-plane form of the two-parameter render at the edges of what the library
+accepts: launch sizes, parameters and data that the scenes of test_gpu_camera_plane.py do
+not have."""
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2308_14737_gb300 import fmb, synth
+
+from gpu_util import dev_scene, gpu_forward
+
+pytestmark = pytest.mark.gpu
+
+WORLD_RAYS = 131072
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2308_14737_gb300 import build
+
+    build.build()
+    oracle.build()
+    fmb.load_library()
+
+
+def _two_views(mu, ch, lam, W=301, H=239):
+    q = lambda x: float(np.float32(x))  # what the library sees
+    poses = [synth.look_at_pose((0.0, 0.0, -4.0)), synth.look_at_pose((2.5, 1.0, 2.5))]
+    views = [dict(W=W, H=H, fx=q(1.1 * W), fy=q(0.9 * W), cx=q(0.4 * W), cy=q(0.6 * H), object=0, pose=i,
+                  flow_target=(1 - i, i)) for i in range(2)]
+    s = synth.make_scene([(mu, ch, lam)], views, poses)
+    assert s.n_pixels > WORLD_RAYS
+    return s
+
+
+@pytest.mark.parametrize("normals,colors,tile", [(1, 0, 430), (0, 0, 753), (0, 1, 502)])
+def test_ray_tiles_whose_shared_memory_ends_at_48_kb(normals, colors, tile):
+    """Dynamic shared memory of 48 160 to 48 192 bytes, which only the static part carries
+    past 48 KB: the gradients of the default tile, whose sums have another order (3e-5)."""
+    K = 40
+    rng = np.random.default_rng(2)
+    s = _two_views(*synth.random_gaussians(rng, K))
+    x = dev_scene(s)
+    P = s.n_pixels
+    T = lambda a: torch.as_tensor(a.reshape(-1), device="cuda")
+    col = torch.rand(K, 3, device="cuda") if colors else None
+    got, ups = [], None
+    for t in (0, tile):
+        params = fmb.default_params(n_flow=2, want_normals=normals, colors=colors, bwd_ray_tile=t)
+        r = fmb.Renderer(s.obj_offsets, s.views, len(s.poses), params)
+        out = r.forward(*x, colors=col)
+        if ups is None:
+            on = (out["alpha"] >= 1e-2).cpu().numpy()
+            gd, ga, gn, gf = synth.upstream_grads(rng, P, 2)
+            ups = [T(gd * on), T(ga), torch.zeros(3 * P, device="cuda"), T(gf * on)]
+        got.append(r.backward(*x, *ups, colors=col, g_color=T(gn * on) if colors else None))
+    for k, t in got[0].items():
+        assert (got[1][k].double() - t.double()).abs().max() <= 3e-5 * t.abs().max(), k
