@@ -32,11 +32,14 @@ namespace fmb {
 // [B10, B11], [e0, e1, e2]] is the root in the frame of the offsets (dx, dy, 1).
 //   0 -pe_x  1 -pe_y   expansion pixel, negated
 //   2 B00  3 B10  4 z  5 d0  6 e0  7 B11  8 e1  9 z B11  10 d1
-//   11 e2^2  12 -log2(lambda)  13 unused  14 rho_x  15 rho_y (m - z c_e, in pixels)
+//   11 e2^2  12 -log2(lambda)  13 flags (bits)  14 rho_x  15 rho_y (m - z c_e, in pixels)
 // An object's last record of an odd count holds its last Gaussian twice, the copy
-// with the log-density -1e30: its weight and density are exactly 0.
+// with the log-density -1e30, so that its density is exactly 0, and flagged
+// kCamCopy: the forward leaves its weight out.  (Its weight's exponent passes through
+// beta1, which may be 0 or negative.  The adjoint's sums of its lane are not read.)
 constexpr int kCamF2 = 16;
 constexpr float kDummyNl2 = 1e30f;
+constexpr int kCamCopy = 2;
 
 // sqrt(log2(e) / 2), its square, and 2 ln 2 (the derivative of d = ln(delta) with
 // respect to a scaled u is -2 ln 2 u).
@@ -46,6 +49,7 @@ constexpr float kTwoLn2 = 1.3862943611198906f;
 
 struct CamRec2 {
   f2 npx, npy, B00, B10, z, d0, e0, B11, e1, F11, d1, ee, nl2;
+  unsigned long long flags;  // of the two Gaussians, one per half
 };
 __device__ __forceinline__ CamRec2 cam_load(const ulonglong2* __restrict__ r) {
   const ulonglong2 q0 = r[0], q1 = r[1], q2 = r[2], q3 = r[3], q4 = r[4], q5 = r[5], q6 = r[6];
@@ -63,6 +67,7 @@ __device__ __forceinline__ CamRec2 cam_load(const ulonglong2* __restrict__ r) {
   g.d1 = as_f2(q5.x);
   g.ee = as_f2(q5.y);
   g.nl2 = as_f2(q6.x);
+  g.flags = q6.y;
   return g;
 }
 

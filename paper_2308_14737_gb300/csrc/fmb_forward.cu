@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(128) prologue_cam_kernel(const __grid_constant
   w[10] = -__fmul_rn(b11.h, rho[1].h);
   w[11] = __fmul_rn(S22.h > 0.f ? S22.h : (S22.h == S22.h ? 0.f : S22.h), kCamScale2);
   w[12] = real ? -log2f(s.weights[g]) : kDummyNl2;
-  w[13] = 0.f;
+  w[13] = __int_as_float(real ? 0 : kCamCopy);
   w[14] = rho[0].h;
   w[15] = rho[1].h;
   const bool odd = (i & 1) != 0;
@@ -376,6 +376,10 @@ __device__ __forceinline__ void fwd_record2(RayAcc2<NORMALS, COLOR> (&A)[RPT], c
   FwdPair2 q[RPT];
 #pragma unroll
   for (int r = 0; r < RPT; ++r) q[r] = fwd_pair2<NORMALS, COLOR>(A[r], g, nB1);
+  if (g.flags != 0) {  // the same for the whole CTA
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) q[r].d = pk(lo(q[r].d), -INFINITY);
+  }
   float top = fmaxf(lo(q[0].d), hi(q[0].d));
 #pragma unroll
   for (int r = 1; r < RPT; ++r) top = fmaxf(top, fmaxf(lo(q[r].d), hi(q[r].d)));

@@ -9,7 +9,8 @@ import torch
 import oracle
 from paper_2308_14737_gb300 import fmb, synth
 
-from gpu_util import dev_scene, gpu_forward
+from gpu_util import (compare_forward, compare_grads, dev_scene, gpu_backward, gpu_forward, masked_upstream,
+                      nnorm_batched)
 
 pytestmark = pytest.mark.gpu
 
@@ -60,3 +61,35 @@ def test_ray_tiles_whose_shared_memory_ends_at_48_kb(normals, colors, tile):
         got.append(r.backward(*x, *ups, colors=col, g_color=T(gn * on) if colors else None))
     for k, t in got[0].items():
         assert (got[1][k].double() - t.double()).abs().max() <= 3e-5 * t.abs().max(), k
+
+
+def _mild(K, seed):
+    """Gaussians of 0.5 to 1 radius: whitened distances stay below about 10, so that 32-bit
+    exponents are good to 1e-5 for any sign of beta1."""
+    rng = np.random.default_rng(seed)
+    mu = rng.uniform(-1, 1, (K, 3))
+    d, o = rng.uniform(1.0, 2.0, (K, 3)), rng.normal(0, 0.3, (K, 3))
+    ch = np.stack([d[:, 0], o[:, 0], d[:, 1], o[:, 1], o[:, 2], d[:, 2]], 1)
+    return mu.astype(np.float32), ch.astype(np.float32), rng.uniform(0.5, 1.5, K).astype(np.float32)
+
+
+@pytest.mark.parametrize("beta1", [0.0, -0.5, 0.3])
+@pytest.mark.parametrize("K,opts", [(1, {}), (3, {}), (65, {}), (65, dict(fwd_ksplit=3)), (5, dict(fwd_rays_per_thread=1)),
+                                    (257, dict(want_normals=0, fwd_rays_per_thread=4)), (64, {})])
+def test_beta1_of_any_sign(beta1, K, opts):
+    """beta1 may be any finite number: planes and gradients against the FP64 oracle."""
+    s = _two_views(*_mild(K, K))
+    params = fmb.default_params(n_flow=1, **opts)
+    params.beta1 = beta1
+    b1 = float(params.beta1)
+    normals = bool(params.want_normals)
+    gpu, r, dev = gpu_forward(s, params)
+    ref = oracle.render_scene(s, n_flow=1, beta1=b1)
+    compare_forward(s, gpu, ref, 1, normals)
+    ups = masked_upstream(s, ref["alpha"], 1, nnorm_ref=nnorm_batched(s, ref["saved"]))
+    if not normals:
+        ups["g_normal"] = np.zeros_like(ups["g_normal"])
+    g = gpu_backward(r, dev, ups)
+    refg = oracle.backward_scene(s, ups["g_depth"], ups["g_alpha"], ups["g_normal"] if normals else None, ups["g_flow"],
+                                 n_flow=1, beta1=b1)
+    compare_grads(g, refg)
