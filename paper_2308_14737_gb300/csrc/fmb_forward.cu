@@ -17,6 +17,9 @@ namespace fmb {
 constexpr int kFwdThreads = 128;
 constexpr int kChunk = 256;  // Gaussians per shared-memory stage (16 KB)
 constexpr int kFwdUnroll = 2;  // records per trip (1: 1 to 2.5 % slower)
+// Minus the shift before a lane's first Gaussian.  Finite: the exponent of a Gaussian of
+// weight 0 is -inf, which must leave its weight at 0 (not inf - inf).
+constexpr float kNoShift = 3e38f;
 
 // ------------------------------------------------------------------ prologue
 // The world-frame kernels' records (fmb_world_*.cu, alpha compositing, point export,
@@ -440,7 +443,7 @@ __device__ __noinline__ RayNormal blended_normal_again(const DevView& V, const f
   pixel_ray_dd(V, R, ray_pixel(V, p), vc, v, vl, pxy);
 #pragma unroll
   for (int c = 0; c < 3; ++c) camera_centre_dd(R, tp, c, oh[c], ol[c]);
-  float m = -INFINITY, Sw = 0.f, N0 = 0.f, N1 = 0.f, N2 = 0.f;
+  float m = -kNoShift, Sw = 0.f, N0 = 0.f, N1 = 0.f, N2 = 0.f;
   for (int base = 0; base < V.K; base += 32) {
     const bool in = base + lane < V.K;
     const long long g = V.gauss_off + min(base + lane, V.K - 1);
@@ -647,7 +650,7 @@ __global__ void __launch_bounds__(kFwdThreads)
       a.r01 = dup(r01);
       a.r11 = dup(r11);
     }
-    a.nm = dup(INFINITY);
+    a.nm = dup(kNoShift);
     a.Sw = a.Swt = a.Sd = a.N0 = a.N1 = a.C0 = a.C1 = a.C2 = dup(0.f);
   }
   const f2 nB1 = dup(-k.beta1), tiny = dup(1e-30f), zero2 = dup(0.f);

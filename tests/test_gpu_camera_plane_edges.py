@@ -93,3 +93,40 @@ def test_beta1_of_any_sign(beta1, K, opts):
     refg = oracle.backward_scene(s, ups["g_depth"], ups["g_alpha"], ups["g_normal"] if normals else None, ups["g_flow"],
                                  n_flow=1, beta1=b1)
     compare_grads(g, refg)
+
+
+@pytest.mark.parametrize("zero", [(0,), (1,), (0, 1), (0, 1, 2, 3), (21, 22, 42, 43, 64)])
+@pytest.mark.parametrize("opts", [{}, dict(fwd_ksplit=3), dict(want_normals=0)])
+def test_weights_of_zero(zero, opts):
+    """A Gaussian whose weight underflowed to 0 leaves the planes and the others' gradients
+    what they are without it, wherever it stands (tolerances of two orders of summation)."""
+    K = 65
+    mu, ch, lam = synth.random_gaussians(np.random.default_rng(9), K)
+    mu[32:40] = mu[24:32] + np.float32([0.0, 0.0, 0.3])  # normals that oppose each other
+    keep = np.setdiff1d(np.arange(K), zero)
+    lam0 = lam.copy()
+    lam0[list(zero)] = 0.0
+    params = fmb.default_params(n_flow=1, **opts)
+    got, ups = [], None
+    for s in (_two_views(mu[keep], ch[keep], lam[keep]), _two_views(mu, ch, lam0)):
+        x = dev_scene(s)
+        r = fmb.Renderer(s.obj_offsets, s.views, len(s.poses), params)
+        out = {k: t.clone() for k, t in r.forward(*x).items() if t is not None}
+        on = out["alpha"] >= 1e-2
+        if ups is None:
+            torch.manual_seed(1)
+            ups = [torch.randn(n * s.n_pixels, device="cuda") for n in (1, 1, 3, 2)]
+            ups = [ups[0] * on, ups[1], ups[2] * 0, 0.01 * ups[3] * on.view(2, 1, -1).expand(2, 2, -1).reshape(-1)]
+        got.append((out, r.backward(*x, *ups), on))
+    (a, ga, on), (b, gb, _) = got
+    assert ((a["depth"] - b["depth"]).abs() / a["depth"])[on].max() <= 1e-5
+    assert (a["alpha"] - b["alpha"]).abs().max() <= 2e-6
+    if params.want_normals:
+        nn = a["saved"].view(2, 3, -1)[:, 2]
+        e = (a["normal"] - b["normal"]).view(2, 3, -1).abs().amax(1) * nn.clamp(min=1e-3)
+        assert e.reshape(-1)[on].max() <= 2e-5
+    assert torch.isfinite(b["normal"]).all() if params.want_normals else True
+    idx = torch.as_tensor(keep, device="cuda")
+    for k in ("means", "chol", "weights"):
+        t = ga[k]
+        assert (gb[k][idx].double() - t.double()).abs().max() <= 3e-5 * t.abs().max(), k
