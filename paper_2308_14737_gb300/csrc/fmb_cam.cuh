@@ -98,7 +98,7 @@ __device__ __forceinline__ CamGeom2 cam_geom2(const CamRec2& g, f2 X, f2 Y) {
 // Reciprocal, reciprocal square root and square root to about an ulp from the MUFU
 // approximation and one Newton step (3 to 5 instructions; the IEEE forms take 10 to 20,
 // and the per-ray code of K = 100 was a quarter of the forward's instructions with
-// them).  For normal, positive arguments; explicitly rounded, so that the forward and
+// them).  For normal, positive, finite arguments (0 and infinity give NaN); explicitly rounded, so that the forward and
 // the adjoint (compiled with different flags) get the same bits.
 __device__ __forceinline__ float rcp_nr(float x) {
   const float r = rcp_approx(x);

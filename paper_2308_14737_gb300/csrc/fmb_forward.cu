@@ -561,7 +561,7 @@ __device__ __forceinline__ void write_ray_outputs(const DevView& V, const float 
         const float X0 = fmaf(Rj[j][2], pt[2], fmaf(Rj[j][1], pt[1], fmaf(Rj[j][0], pt[0], tj[j][0])));
         const float X1 = fmaf(Rj[j][5], pt[2], fmaf(Rj[j][4], pt[1], fmaf(Rj[j][3], pt[0], tj[j][1])));
         const float X2 = fmaf(Rj[j][8], pt[2], fmaf(Rj[j][7], pt[1], fmaf(Rj[j][6], pt[0], tj[j][2])));
-        const float iz = rcp_nr(X2);
+        const float iz = 1.0f / X2;  // not rcp_nr: a point in the target's camera plane has infinite flow
         fu = fmaf(V.fx * X0, iz, V.cx) - ray.px;
         fv = fmaf(V.fy * X1, iz, V.cy) - ray.py;
       }

@@ -130,3 +130,20 @@ def test_weights_of_zero(zero, opts):
     for k in ("means", "chol", "weights"):
         t = ga[k]
         assert (gb[k][idx].double() - t.double()).abs().max() <= 3e-5 * t.abs().max(), k
+
+
+def test_flow_of_points_in_the_targets_camera_plane():
+    """One flat Gaussian facing the camera, seen at depth 4 on every ray, and a target camera
+    whose plane holds it: the flow is infinite, with the sign of the point's offset."""
+    W, H = 401, 331
+    mu, ch = np.array([[0.0, 0.0, 4.0]], np.float32), np.array([[1e-3, 0, 1e-3, 0, 0, 100.0]], np.float32)
+    pose = np.concatenate([np.eye(3).reshape(-1), [0, 0, 0]])
+    target = np.concatenate([np.eye(3).reshape(-1), [0, 0, -4.0]])
+    view = dict(W=W, H=H, fx=300.0, fy=300.0, cx=200.25, cy=165.25, object=0, pose=0, flow_target=(1, -1))
+    s = synth.make_scene([(mu, ch, np.ones(1, np.float32))], [view], [pose, target])
+    assert s.n_pixels > WORLD_RAYS
+    gpu, _, _ = gpu_forward(s, fmb.default_params(n_flow=1, want_normals=0))
+    f = gpu["flow"].reshape(2, H, W)
+    x, y = np.arange(W) + 0.5 - 200.25, np.arange(H) + 0.5 - 165.25
+    np.testing.assert_array_equal(f[0], np.broadcast_to(np.copysign(np.inf, x), (H, W)))
+    np.testing.assert_array_equal(f[1], np.broadcast_to(np.copysign(np.inf, y)[:, None], (H, W)))
