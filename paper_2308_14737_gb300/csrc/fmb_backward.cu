@@ -91,7 +91,8 @@ __host__ __device__ constexpr int ray_rec2() {
   return 4 + (NORMALS ? 3 : 0) + (COLOR ? 2 : 0);
 }
 
-template <bool NORMALS, bool COLOR, bool POSE>
+// FLAT: a warp with flat Gaussians (cam_flat_flags).
+template <bool NORMALS, bool COLOR, bool POSE, bool FLAT>
 __device__ __forceinline__ void bwd_pair2(BwdAcc2<NORMALS, COLOR, POSE>& S, const CamRec2& g,
                                           const ulonglong2* __restrict__ rr, f2 nB1, f2 nB1s, f2 tiny, f2 c0,
                                           f2 c1, f2 c2) {
@@ -99,7 +100,7 @@ __device__ __forceinline__ void bwd_pair2(BwdAcc2<NORMALS, COLOR, POSE>& S, cons
   const ulonglong2 q0 = rr[0], q1 = rr[1], q2 = rr[2], q3 = rr[3];
   const f2 nlse = as_f2(q1.x), K2 = as_f2(q1.y), Dbar = as_f2(q2.x), nD = as_f2(q2.y), nKA = as_f2(q3.x),
            nB2E = as_f2(q3.y);
-  const CamGeom2 G = cam_geom2(g, as_f2(q0.x), as_f2(q0.y));
+  const CamGeom2 G = cam_geom2<FLAT && NORMALS>(g, as_f2(q0.x), as_f2(q0.y));
   const f2 what = ex2_2(fma2(G.t, K2, fma2(G.nx, nB1, nlse)));
   const f2 delta = pk(ex2_approx(-lo(G.nx)), ex2_approx(-hi(G.nx)));
   const f2 Dw = mul2(Dbar, what), tD = add2(G.t, nD);
@@ -504,9 +505,11 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
   Acc A;
 #pragma unroll
   for (int i = 0; i < Acc::kN; ++i) A.v[i] = dup(0.f);
+  const long long rec0 = static_cast<long long>(V.rec_off) + (active ? g0 : 0);
+  const CamRec2 gr = cam_load(reinterpret_cast<const ulonglong2*>(records + kRecFloat4 * rec0));
+  constexpr unsigned long long kFlat = (static_cast<unsigned long long>(kCamFlatter) << 32) | kCamFlatter;
+  const bool flat = NORMALS && __any_sync(0xffffffffu, active && (gr.flags & kFlat) != 0);
   if (active) {
-    const long long rec0 = static_cast<long long>(V.rec_off) + g0;
-    const CamRec2 gr = cam_load(reinterpret_cast<const ulonglong2*>(records + kRecFloat4 * rec0));
     const f2 nB1 = dup(-k.beta1), nB1s = dup(-kTwoLn2 * k.beta1), tiny = dup(-1e-30f);
     const ulonglong2* rays = reinterpret_cast<const ulonglong2*>(bsm);
     constexpr int NR = ray_rec2<NORMALS, COLOR>(), kUnroll = bwd_unroll<NORMALS>();
@@ -517,9 +520,15 @@ __global__ void __launch_bounds__(kBwdMaxThreads, kBwdMinBlocks)
       c1 = as_f2(cr[0].y);
       c2 = as_f2(cr[1].x);
     }
+    if (!flat) {
 #pragma unroll kUnroll
-    for (int r = sg; r < nr; r += S)
-      bwd_pair2<NORMALS, COLOR, POSE>(A, gr, rays + NR * r, nB1, nB1s, tiny, c0, c1, c2);
+      for (int r = sg; r < nr; r += S)
+        bwd_pair2<NORMALS, COLOR, POSE, false>(A, gr, rays + NR * r, nB1, nB1s, tiny, c0, c1, c2);
+    } else if (NORMALS) {
+#pragma unroll 1
+      for (int r = sg; r < nr; r += S)
+        bwd_pair2<NORMALS, COLOR, POSE, NORMALS>(A, gr, rays + NR * r, nB1, nB1s, tiny, c0, c1, c2);
+    }
   }
   __syncthreads();  // ray records are dead; the shared memory is reused below
 

@@ -13,7 +13,7 @@
 // The pixel offsets from c_e are exact near the projection (Sterbenz) and m - z c_e
 // is formed in float pairs, so u keeps its relative accuracy for rays that pass close
 // to a distant mean, where t a - b in plain fp32 loses |b|/|u| ulps.  25 operations
-// per pair without the normal, 36 with it; the world-frame evaluation (exact float
+// per pair without the normal, 36 with it (42 for flat Gaussians, cam_flat_flags); the world-frame evaluation (exact float
 // pairs of the ray and of mu - o, and a second projection of u) took 35 and 56 at the
 // same error (log-weights 1.0-2.1e-6 rms against 1.3-2.2e-6, FP64 comparison on the
 // benchmark's scenes).
@@ -37,9 +37,29 @@ namespace fmb {
 // with the log-density -1e30, so that its density is exactly 0, and flagged
 // kCamCopy: the forward leaves its weight out.  (Its weight's exponent passes through
 // beta1, which may be 0 or negative.  The adjoint's sums of its lane are not read.)
+// kCamFlat, kCamFlatter: see cam_flat_flags.
 constexpr int kCamF2 = 16;
 constexpr float kDummyNl2 = 1e30f;
-constexpr int kCamCopy = 2;
+constexpr int kCamFlat = 1, kCamCopy = 2, kCamFlatter = 4;
+
+// The rounding of tau leaves a component dtau a in u, to which u . u is stationary but
+// the normal g = B u is not: it moves by dtau P c, and |P c| exceeds |g| by up to the
+// square of the axis ratio.  A second projection of u onto the complement of a (6
+// operations) takes it out.  Only flat Gaussians need it.  With l1 >= l2 >= l3 the axes
+// of the root, tr(P)^2 over the sum of P's principal 2x2 minors is about (l1/l2)^2 / 2
+// (thin discs) and tr(P) tr(P^-1) about 2 (l1/l3)^2 (needles too).  Normals of discs
+// (sigma 0.4, depth 4, rms against FP64; projected / not): ratio 3 0.8e-7 / 0.7e-7, 6 1.1e-7 /
+// 2.0e-7, 10 1.4e-7 / 5.1e-7, 30 1.7e-7 / 4.4e-6, 100 1.7e-7 / 4.9e-5, growing with the square:
+// the forward projects from a ratio of 5 on (4 % of the benchmark's Gaussians).  The
+// gradients were within the projected form's up to a ratio of 30 (L: 1.1e-5 / 1.8e-5) and
+// past it at 100 (1.2e-4 / 0.9e-5): the adjoint, whose warps hold 64 Gaussians each, projects
+// from 16 on.  Both rules cost the benchmark's scenes 0 to 0.8 % (orbit 648.6 -> 650.8 us,
+// 1023x767 at K = 333 358 -> 361).
+__device__ __forceinline__ int cam_flat_flags(float trace, float minors, float det) {
+  const bool needle = !(trace * minors < 1000.f * det);
+  return (needle || !(trace * trace < 14.f * minors) ? kCamFlat : 0) |
+         (needle || !(trace * trace < 130.f * minors) ? kCamFlatter : 0);
+}
 
 // sqrt(log2(e) / 2), its square, and 2 ln 2 (the derivative of d = ln(delta) with
 // respect to a scaled u is -2 ln 2 u).
@@ -76,6 +96,7 @@ struct CamGeom2 {
   f2 dx, dy, a0, a1, ninv, tau, t, u0, u1, nx;  // ninv = -1 / a.a;  nx = -log2(delta)
 };
 __device__ __forceinline__ f2 rcp_neg_2(f2 a) { return pk(rcp_approx(-lo(a)), rcp_approx(-hi(a))); }
+template <bool PROJECT = false>  // the second projection of u (see cam_flat_flags)
 __device__ __forceinline__ CamGeom2 cam_geom2(const CamRec2& g, f2 X, f2 Y) {
   CamGeom2 G;
   G.dx = add2(X, g.npx);
@@ -92,6 +113,11 @@ __device__ __forceinline__ CamGeom2 cam_geom2(const CamRec2& g, f2 X, f2 Y) {
   G.u0 = fma2(G.tau, G.a0, D0);
   G.u1 = fma2(G.tau, G.a1, D1);
   G.nx = fma2(G.u0, G.u0, fma2(G.u1, G.u1, fma2(mul2(G.tau, G.tau), g.ee, g.nl2)));
+  if (PROJECT) {
+    const f2 nk = mul2(fma2(G.u0, G.a0, fma2(G.u1, G.a1, mul2(G.tau, g.ee))), G.ninv);
+    G.u0 = fma2(nk, G.a0, G.u0);
+    G.u1 = fma2(nk, G.a1, G.u1);
+  }
   return G;
 }
 

@@ -16,7 +16,6 @@ namespace fmb {
 
 constexpr int kFwdThreads = 128;
 constexpr int kChunk = 256;  // Gaussians per shared-memory stage (16 KB)
-constexpr int kFwdUnroll = 2;  // records per trip (1: 1 to 2.5 % slower)
 // Minus the shift before a lane's first Gaussian.  Finite: the exponent of a Gaussian of
 // weight 0 is -inf, which must leave its weight at 0 (not inf - inf).
 constexpr float kNoShift = 3e38f;
@@ -225,7 +224,10 @@ __global__ void __launch_bounds__(128) prologue_cam_kernel(const __grid_constant
   w[10] = -__fmul_rn(b11.h, rho[1].h);
   w[11] = __fmul_rn(S22.h > 0.f ? S22.h : (S22.h == S22.h ? 0.f : S22.h), kCamScale2);
   w[12] = real ? -log2f(s.weights[g]) : kDummyNl2;
-  w[13] = __int_as_float(real ? 0 : kCamCopy);
+  const FF m2 = P00 * P(1, 1) - P(1, 0) * P(1, 0) + P00 * P(2, 2) - P(2, 0) * P(2, 0) + P(1, 1) * P(2, 2) -
+                P(2, 1) * P(2, 1);
+  w[13] = __int_as_float((real ? 0 : kCamCopy) |
+                         cam_flat_flags((P00 + P(1, 1) + P(2, 2)).h, m2.h, P00.h * S11.h * S22.h));
   w[14] = rho[0].h;
   w[15] = rho[1].h;
   const bool odd = (i & 1) != 0;
@@ -311,9 +313,9 @@ __device__ __forceinline__ void ray_metric(const DevView& V, const CamRay& r, fl
 struct FwdPair2 {
   f2 d, t, nx, u0, u1;
 };
-template <bool NORMALS, bool COLOR>
+template <bool NORMALS, bool COLOR, bool FLAGGED>
 __device__ __forceinline__ FwdPair2 fwd_pair2(RayAcc2<NORMALS, COLOR>& A, const CamRec2& g, f2 nB1) {
-  const CamGeom2 G = cam_geom2(g, A.X, A.Y);
+  const CamGeom2 G = cam_geom2<FLAGGED && NORMALS>(g, A.X, A.Y);
   A.Sd = add2(A.Sd, pk(ex2_approx(-lo(G.nx)), ex2_approx(-hi(G.nx))));
   return FwdPair2{fma2(G.t, A.K2, fma2(G.nx, nB1, A.nm)), G.t, G.nx, G.u0, G.u1};
 }
@@ -372,16 +374,18 @@ __device__ __forceinline__ void fwd_sum2(RayAcc2<NORMALS, COLOR>& A, const CamRe
 }
 
 // One record against the thread's rays, with one check of the shifts for all of them (a
-// check per ray cost 6 to 9 % of the kernel).
-template <int RPT, bool NORMALS, bool COLOR>
+// check per ray cost 6 to 9 % of the kernel).  FLAGGED: a record with a flat Gaussian (with
+// normals) or a copy.
+template <int RPT, bool NORMALS, bool COLOR, bool FLAGGED>
 __device__ __forceinline__ void fwd_record2(RayAcc2<NORMALS, COLOR> (&A)[RPT], const CamRec2& g, f2 nB1, f2 tiny, f2 c0,
                                             f2 c1, f2 c2) {
   FwdPair2 q[RPT];
 #pragma unroll
-  for (int r = 0; r < RPT; ++r) q[r] = fwd_pair2<NORMALS, COLOR>(A[r], g, nB1);
-  if (g.flags != 0) {  // the same for the whole CTA
+  for (int r = 0; r < RPT; ++r) q[r] = fwd_pair2<NORMALS, COLOR, FLAGGED>(A[r], g, nB1);
+  if (FLAGGED) {
+    const bool copy = (g.flags >> 32 & kCamCopy) != 0;
 #pragma unroll
-    for (int r = 0; r < RPT; ++r) q[r].d = pk(lo(q[r].d), -INFINITY);
+    for (int r = 0; r < RPT; ++r) q[r].d = pk(lo(q[r].d), copy ? -INFINITY : hi(q[r].d));
   }
   float top = fmaxf(lo(q[0].d), hi(q[0].d));
 #pragma unroll
@@ -578,8 +582,18 @@ __host__ __device__ constexpr int fwd_stage_float4() {
   return kChunk * (kRecFloat4 + (COLOR ? 1 : 0));
 }
 
+// Resident CTAs per SM the register budget keeps where the compiler, with the code for
+// flagged records beside the plain one, would take more than 168 registers (four rays per
+// thread: 220, orbit render and adjoint 661 against 654 us) or 128 (normals and flow: 157).
+// The others are left alone: a bound of 4 took 128 registers instead of 118 for normals
+// without flow and was slower (1023x767 at K = 333 382 against 362 us).
+template <bool NORMALS, int NFLOW, int RPT, bool COLOR>
+constexpr int fwd_min_blocks() {
+  return COLOR ? 0 : (RPT == 4 ? 3 : (RPT == 2 && NORMALS && NFLOW > 0 ? 4 : 0));
+}
+
 template <bool NORMALS, int NFLOW, int RPT, bool COLOR = false, class B = Batch>
-__global__ void __launch_bounds__(kFwdThreads)
+__global__ void __launch_bounds__(kFwdThreads, fwd_min_blocks<NORMALS, NFLOW, RPT, COLOR>())
     forward_kernel(const __grid_constant__ B batch, Scene s,
                                                               Consts k, const float4* __restrict__ records,
                                                               FwdOut out, int* status, int* counter) {
@@ -654,6 +668,9 @@ __global__ void __launch_bounds__(kFwdThreads)
     a.Sw = a.Swt = a.Sd = a.N0 = a.N1 = a.C0 = a.C1 = a.C2 = dup(0.f);
   }
   const f2 nB1 = dup(-k.beta1), tiny = dup(1e-30f), zero2 = dup(0.f);
+  // what takes a record through the longer code (the same for the whole CTA)
+  constexpr unsigned long long kFlags = (static_cast<unsigned long long>(kCamCopy | (NORMALS ? kCamFlat : 0)) << 32) |
+                                        (NORMALS ? kCamFlat : 0);
 
   bool failed = false;
   for (int c = 0; c < nchunks; ++c) {
@@ -667,17 +684,35 @@ __global__ void __launch_bounds__(kFwdThreads)
     const int n = min(kChunk, K - c * kChunk);
     const ulonglong2* rec = reinterpret_cast<const ulonglong2*>(fwd_smem + stage * SST);
     const ulonglong2* crs = rec + kChunk * kRecFloat4;  // colour mode: this stage's colour records
-#pragma unroll kFwdUnroll
-    for (int i = 0; i < n; i += 2) {
-      const CamRec2 g = cam_load(rec + kRecFloat4 * i);
-      f2 c0 = zero2, c1 = zero2, c2 = zero2;
+    auto color_of = [&](int i, f2& c0, f2& c1, f2& c2) {
+      c0 = c1 = c2 = zero2;
       if (COLOR) {
         const ulonglong2 q0 = crs[i], q1 = crs[i + 1];
         c0 = as_f2(q0.x);
         c1 = as_f2(q0.y);
         c2 = as_f2(q1.x);
       }
-      fwd_record2<RPT, NORMALS, COLOR>(A, g, nB1, tiny, c0, c1, c2);
+    };
+    int i = 0;
+    while (i < n) {
+      // two plain records per trip (one: 1 to 2.5 % slower), up to the first flagged one
+      for (; i + 2 < n; i += 4) {
+        const CamRec2 g = cam_load(rec + kRecFloat4 * i), h = cam_load(rec + kRecFloat4 * (i + 2));
+        if (((g.flags | h.flags) & kFlags) != 0) break;
+        f2 c0, c1, c2;
+        color_of(i, c0, c1, c2);
+        fwd_record2<RPT, NORMALS, COLOR, false>(A, g, nB1, tiny, c0, c1, c2);
+        color_of(i + 2, c0, c1, c2);
+        fwd_record2<RPT, NORMALS, COLOR, false>(A, h, nB1, tiny, c0, c1, c2);
+      }
+      // and the next two, or the last one, by the longer code
+      const int end = min(i + 4, n);
+#pragma unroll 1
+      for (; i < end; i += 2) {
+        f2 c0, c1, c2;
+        color_of(i, c0, c1, c2);
+        fwd_record2<RPT, NORMALS, COLOR, true>(A, cam_load(rec + kRecFloat4 * i), nB1, tiny, c0, c1, c2);
+      }
     }
     __syncthreads();  // every thread is done with this stage before it is refilled
     if (tid == 0 && c + 2 < nchunks) {
