@@ -7,6 +7,7 @@
 //   [256, 256 + 64 R)   R per-(view, Gaussian) records, R = sum over views of K, each
 //                       view's K rounded up to an even count
 //   [.., ..)            backward partials (deterministic mode and the camera-plane form)
+//   and what workspace_needed lists after them
 #include <algorithm>
 #include <cmath>
 #include <cstddef>
@@ -461,7 +462,8 @@ Plan make_plan(const fmb_params* p, const long long* offs, int n_objects, int n_
 
 // Workspace: header (status word, work counters) | records | colour records (if
 // colors) | partial sums (if deterministic, or in the camera-plane form) | per-pair t, e2, delta
-// arrays (if store_pairs).
+// arrays (if store_pairs) | split forward's sums | depth orders (if keep_order) | the
+// adjoint's second records (camera-plane form).
 size_t crec_offset(const Plan& pl) {
   return kHeaderBytes + align256(static_cast<size_t>(pl.n_records) * 16 * fmb::kRecFloat4);
 }
@@ -490,7 +492,13 @@ size_t order_bytes(const fmb_params* p, const Plan& pl) {
   return align256(static_cast<size_t>(pl.n_entries) * 32 * fmb::ac_lanes_per_ray_elements(pl.maxK));
 }
 
-size_t workspace_needed(const fmb_params* p, const Plan& pl) { return order_offset(p, pl) + order_bytes(p, pl); }
+// The camera-plane adjoint's second records (Scene::qrec), last.
+size_t qrec_offset(const fmb_params* p, const Plan& pl) { return order_offset(p, pl) + order_bytes(p, pl); }
+
+size_t workspace_needed(const fmb_params* p, const Plan& pl) {
+  const bool cam = p->variant == 0 && !pl.world;
+  return qrec_offset(p, pl) + (cam ? align256(static_cast<size_t>(pl.n_records) * 16 * fmb::kCamQFloat4) : 0);
+}
 
 fmb::Consts make_consts(const fmb_params* p) {
   const double log2e = 1.4426950408889634;
@@ -717,6 +725,7 @@ fmb_status fmb_render_backward(const fmb_params* params, int n_objects, const lo
       sc.colors = colors;
       sc.crec = reinterpret_cast<float4*>(base + crec_offset(pl));
     }
+    if (params->variant == 0 && !pl.world) sc.qrec = reinterpret_cast<float4*>(base + qrec_offset(params, pl));
     const fmb::Consts c = make_consts(params);
     const bool normals = params->want_normals != 0;
     const float* pairs =

@@ -31,9 +31,9 @@
 // sigma = s - dbar tau and kappa = tau (sigma + s) alone (abar_2 = kappa e2,
 // y_2 = sigma e2).  The render depends on B only through P = B B^T, so the gradient
 // with respect to a full 3x3 root is X B with X symmetric (X = 2 Pbar), and the six
-// lower entries that are accumulated give X by substitution; then Lbar =
-// lower(R^T X A) and Rbar = X A L^T with A = R L, and the mean's gradient comes from
-// sum y.  Ten sums per Gaussian instead of the nineteen of the world-frame form, and with
+// lower entries that are accumulated give X, and with it the three upper ones, by
+// substitution; then with A = R L Lbar = lower(R^T (X B) (B^-1 A)) and Rbar =
+// (X B) B^T R^-T, and the mean's gradient comes from sum y.  Ten sums per Gaussian instead of the nineteen of the world-frame form, and with
 // normals and pose gradients five more (below).
 #include <algorithm>
 
@@ -185,11 +185,18 @@ __device__ __forceinline__ float warp_sum(float x) {
   return x;
 }
 
-// A Gaussian's gradients from its summed accumulators: X of the header from the lower
-// entries of X B' in the offsets' frame, brought to the camera frame (c = S c', S =
-// [[1/fx, 0, xe], [0, 1/fy, ye], [0, 0, 1]]), then Lbar = lower(R^T X A), mubar = R^-1
-// mbar, and the pose: Rbar = X A L^T - (R^-T mu) mubar^T (+ the normal's term), tbar =
-// mbar, as functions of a general R (A = R L, m = R^-T mu + t).
+// A Gaussian's gradients from its summed accumulators, X B of the header first: M = X B'
+// in the offsets' frame (c = S c', S = [[1/fx, 0, xe], [0, 1/fy, ye], [0, 0, 1]]), whose
+// lower entries were accumulated.  Then X B = S M, Lbar = lower(R^T (X B) Q) with Q =
+// B^-1 A from the prologue, mubar = R^-1 mbar, and the pose: Rbar = (X B) B^T R^-T -
+// (R^-T mu) mubar^T (+ the normal's term), tbar = mbar, as functions of a general R (A =
+// R L, m = R^-T mu + t).
+// X itself, times A, would be the same, but its rounding is multiplied by the axis ratio
+// there, while the columns of M along the short axes were summed directly.  The upper
+// entry M01 still cancels for needles: flat Gaussians take it in float pairs.
+// Discs, alpha's upstream alone, K = 24, against FP64 (world-frame form / X A / now):
+// poses at ratio 100 2.4e-6 / 8.6e-5 / 1.5e-6, at 1000 3.6e-6 / 5.3e-3 / 3.4e-6; L at 1000 2.0e-6 /
+// 5.4e-5 / 5.5e-7.  Orbit 650.8 -> 655 us, 9 views of 257x191 with colours 166 -> 168.6.
 template <bool NORMALS, bool COLOR, bool POSE>
 __device__ __forceinline__ void bwd_finalise(const Scene& s, const DevView& V, const float4* __restrict__ records,
                                              const float* view_inv, int g, const float* acc, bool want_pose, float gm[3],
@@ -206,38 +213,41 @@ __device__ __forceinline__ void bwd_finalise(const Scene& s, const DevView& V, c
   const float b20 = acc[6], b21 = acc[7];
   const float i0 = B00 != 0.f ? 1.0f / B00 : 0.f, i1 = B11 != 0.f ? 1.0f / B11 : 0.f;
   const float X22 = Kp;
-  const float X21 = fmaf(-X22, e1, b21) * i1;
-  const float X11 = fmaf(-X21, e1, b11) * i1;
-  const float X20 = fmaf(-X22, e0, fmaf(-X21, B10, b20)) * i0;
-  const float X10 = fmaf(-X21, e0, fmaf(-X11, B10, b10)) * i0;
-  const float X00 = fmaf(-X20, e0, fmaf(-X10, B10, b00)) * i0;
-  // camera frame: S X S^T, with the scale of the whitened quantities
+  float X21, X20, M01;
+  if ((__float_as_int(rec[26]) & kCamFlatter) == 0) {
+    X21 = fmaf(-X22, e1, b21) * i1;
+    const float X11 = fmaf(-X21, e1, b11) * i1;
+    X20 = fmaf(-X22, e0, fmaf(-X21, B10, b20)) * i0;
+    const float X10 = fmaf(-X21, e0, fmaf(-X11, B10, b10)) * i0;
+    M01 = fmaf(X10, B11, X20 * e1);
+  } else {
+    const FF j0 = B00 != 0.f ? ff_rcp(FF{B00, 0.f}) : FF{0.f, 0.f}, j1 = B11 != 0.f ? ff_rcp(FF{B11, 0.f}) : FF{0.f, 0.f};
+    const FF Y21 = (FF{b21, 0.f} - ff_prod(X22, e1)) * j1;
+    const FF Y11 = (FF{b11, 0.f} - Y21 * e1) * j1;
+    const FF Y20 = (FF{b20, 0.f} - ff_prod(X22, e0) - Y21 * B10) * j0;
+    const FF Y10 = (FF{b10, 0.f} - Y11 * B10 - Y21 * e0) * j0;
+    X21 = Y21.h;
+    X20 = Y20.h;
+    M01 = (Y10 * B11 + Y20 * e1).h;
+  }
+  const float e2 = sqrtf(ee);
+  const float M[9] = {b00, M01, X20 * e2, b10, b11, X21 * e2, b20, b21, X22 * e2};
   const float ifx = 1.0f / V.fx, ify = 1.0f / V.fy, px = pex - V.cx, py = pey - V.cy;
   const float xe = px * ifx, ye = py * ify;
-  const float t0 = X20 * ifx, t1 = X21 * ify;
-  float X[9];
-  X[8] = kCamScale2 * X22;
-  X[6] = kCamScale2 * fmaf(xe, X22, t0);
-  X[7] = kCamScale2 * fmaf(ye, X22, t1);
-  X[0] = fmaf(kCamScale2, fmaf(X00 * ifx, ifx, xe * t0), xe * X[6]);
-  X[4] = fmaf(kCamScale2, fmaf(X11 * ify, ify, ye * t1), ye * X[7]);
-  X[1] = fmaf(kCamScale2, fmaf(X10 * ifx, ify, xe * t1), ye * X[6]);
-  X[2] = X[6];
-  X[3] = X[1];
-  X[5] = X[7];
   float R[9], tp[3];
   load_pose(s.poses, V.pose, R, tp);
-  const float* Lp = s.chol + 6 * gg;
-  const float L00 = Lp[0], L10 = Lp[1], L11 = Lp[2], L20 = Lp[3], L21 = Lp[4], L22 = Lp[5];
-  float XA[9];  // X A = Abar
+  const float4* qr = s.qrec + kCamQFloat4 * (static_cast<long long>(V.rec_off) + g);
+  const float4 qa = qr[0], qb = qr[1], qc = qr[2];
+  const float Q[9] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w, qc.x};
+  float XA[9];  // (X B) Q
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    float XR[3];
+    float XB[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) XR[c] = fmaf(X[3 * a + 2], R[6 + c], fmaf(X[3 * a + 1], R[3 + c], X[3 * a] * R[c]));
-    XA[3 * a + 0] = fmaf(XR[2], L20, fmaf(XR[1], L10, XR[0] * L00));
-    XA[3 * a + 1] = fmaf(XR[2], L21, XR[1] * L11);
-    XA[3 * a + 2] = XR[2] * L22;
+    for (int c = 0; c < 3; ++c)
+      XB[c] = kCamScale * (a == 0 ? fmaf(ifx, M[c], xe * M[6 + c]) : a == 1 ? fmaf(ify, M[3 + c], ye * M[6 + c]) : M[6 + c]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) XA[3 * a + c] = fmaf(XB[2], Q[6 + c], fmaf(XB[1], Q[3 + c], XB[0] * Q[c]));
   }
   auto RtXA = [&](int a, int c) { return fmaf(R[6 + a], XA[6 + c], fmaf(R[3 + a], XA[3 + c], R[a] * XA[c])); };
   gL[0] = RtXA(0, 0);
@@ -269,15 +279,32 @@ __device__ __forceinline__ void bwd_finalise(const Scene& s, const DevView& V, c
     T[5] = T[7] = -V.fy * V1;
     T[8] = -(T[0] + T[4]);
   }
+  // (X B) B^T in the camera frame: S (M B'^T) S^-1
+  float W[9], G[9];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    W[3 * a] = M[3 * a] * B00;
+    W[3 * a + 1] = fmaf(M[3 * a + 1], B11, M[3 * a] * B10);
+    W[3 * a + 2] = fmaf(M[3 * a + 2], e2, fmaf(M[3 * a + 1], e1, M[3 * a] * e0));
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    float u[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      u[c] = a == 0 ? fmaf(ifx, W[c], xe * W[6 + c]) : a == 1 ? fmaf(ify, W[3 + c], ye * W[6 + c]) : W[6 + c];
+    G[3 * a] = u[0] * V.fx;
+    G[3 * a + 1] = u[1] * V.fy;
+    G[3 * a + 2] = fmaf(-px, u[0], fmaf(-py, u[1], u[2]));
+  }
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     // row a of R^-T mu
     const float rm = fmaf(view_inv[6 + a], mu2, fmaf(view_inv[3 + a], mu1, view_inv[a] * mu0));
-    float row[3] = {XA[3 * a] * L00, fmaf(XA[3 * a + 1], L11, XA[3 * a] * L10),
-                    fmaf(XA[3 * a + 2], L22, fmaf(XA[3 * a + 1], L21, XA[3 * a] * L20))};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      float x = fmaf(-rm, gm[c], row[c]);
+      float x = fmaf(-rm, gm[c], fmaf(G[3 * a + 2], view_inv[3 * c + 2],
+                                      fmaf(G[3 * a + 1], view_inv[3 * c + 1], G[3 * a] * view_inv[3 * c])));
       if (NORMALS) x += fmaf(T[3 * a + 2], R[6 + c], fmaf(T[3 * a + 1], R[3 + c], T[3 * a] * R[c]));
       pose_g[3 * a + c] += x;
     }

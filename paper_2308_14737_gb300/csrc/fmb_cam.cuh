@@ -67,6 +67,58 @@ constexpr float kCamScale = 0.84932180028801904f;
 constexpr float kCamScale2 = 0.72134752044448170f;
 constexpr float kTwoLn2 = 1.3862943611198906f;
 
+// Float pairs (unevaluated sums h + l, about 2^-46 relative): the prologue of the
+// camera-plane records forms P = A A^T and its Cholesky factor in them, since P
+// squares the condition of L, and the adjoint solves for a flat Gaussian's gradients.
+// About 900 fp32 instructions per record; FP64 would take fewer, but issues one warp
+// instruction per 16 cycles and SM here.
+struct FF {
+  float h, l;
+};
+__device__ __forceinline__ FF ff_renorm(float h, float l) {
+  const float s = __fadd_rn(h, l);
+  return FF{s, __fsub_rn(l, __fsub_rn(s, h))};
+}
+__device__ __forceinline__ FF operator+(FF a, FF b) {
+  float s, e;
+  two_sum(a.h, b.h, s, e);
+  return ff_renorm(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ FF operator-(FF a) { return FF{-a.h, -a.l}; }
+__device__ __forceinline__ FF operator-(FF a, FF b) { return a + (-b); }
+__device__ __forceinline__ FF operator*(FF a, FF b) {
+  float p, e;
+  two_prod(a.h, b.h, p, e);
+  return ff_renorm(p, fmaf(a.h, b.l, fmaf(a.l, b.h, e)));
+}
+__device__ __forceinline__ FF operator*(FF a, float b) {
+  float p, e;
+  two_prod(a.h, b, p, e);
+  return ff_renorm(p, fmaf(a.l, b, e));
+}
+__device__ __forceinline__ FF ff_prod(float a, float b) {
+  FF r;
+  two_prod(a, b, r.h, r.l);
+  return r;
+}
+__device__ __forceinline__ FF ff_diff(float a, float b) {
+  FF r;
+  two_sum(a, -b, r.h, r.l);
+  return r;
+}
+// 1 / a and 1 / sqrt(a): one Newton step in pair arithmetic from the fp32 value.
+__device__ __forceinline__ FF ff_rcp(FF a) {
+  const float y = __frcp_rn(a.h);
+  const FF r = FF{1.f, 0.f} - a * y;
+  return ff_renorm(y, __fmul_rn(y, r.h));
+}
+__device__ __forceinline__ FF ff_rsqrt(FF a) {  // 0 for a <= 0 (a singular precision)
+  if (!(a.h > 0.f)) return FF{a.h == a.h ? 0.f : a.h, 0.f};
+  const float y = rsqrtf(a.h);
+  const FF r = FF{1.f, 0.f} - a * ff_prod(y, y);
+  return ff_renorm(y, __fmul_rn(0.5f * y, r.h));
+}
+
 struct CamRec2 {
   f2 npx, npy, B00, B10, z, d0, e0, B11, e1, F11, d1, ee, nl2;
   unsigned long long flags;  // of the two Gaussians, one per half

@@ -89,57 +89,6 @@ __global__ void __launch_bounds__(128) prologue_kernel(const __grid_constant__ B
   (void)k;
 }
 
-// Float pairs (unevaluated sums h + l, about 2^-46 relative): the prologue of the
-// camera-plane records forms P = A A^T and its Cholesky factor in them, since P
-// squares the condition of L.  About 900 fp32 instructions per record; FP64 would
-// take fewer, but issues one warp instruction per 16 cycles and SM here.
-struct FF {
-  float h, l;
-};
-__device__ __forceinline__ FF ff_renorm(float h, float l) {
-  const float s = __fadd_rn(h, l);
-  return FF{s, __fsub_rn(l, __fsub_rn(s, h))};
-}
-__device__ __forceinline__ FF operator+(FF a, FF b) {
-  float s, e;
-  two_sum(a.h, b.h, s, e);
-  return ff_renorm(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
-}
-__device__ __forceinline__ FF operator-(FF a) { return FF{-a.h, -a.l}; }
-__device__ __forceinline__ FF operator-(FF a, FF b) { return a + (-b); }
-__device__ __forceinline__ FF operator*(FF a, FF b) {
-  float p, e;
-  two_prod(a.h, b.h, p, e);
-  return ff_renorm(p, fmaf(a.h, b.l, fmaf(a.l, b.h, e)));
-}
-__device__ __forceinline__ FF operator*(FF a, float b) {
-  float p, e;
-  two_prod(a.h, b, p, e);
-  return ff_renorm(p, fmaf(a.l, b, e));
-}
-__device__ __forceinline__ FF ff_prod(float a, float b) {
-  FF r;
-  two_prod(a, b, r.h, r.l);
-  return r;
-}
-__device__ __forceinline__ FF ff_diff(float a, float b) {
-  FF r;
-  two_sum(a, -b, r.h, r.l);
-  return r;
-}
-// 1 / a and 1 / sqrt(a): one Newton step in pair arithmetic from the fp32 value.
-__device__ __forceinline__ FF ff_rcp(FF a) {
-  const float y = __frcp_rn(a.h);
-  const FF r = FF{1.f, 0.f} - a * y;
-  return ff_renorm(y, __fmul_rn(y, r.h));
-}
-__device__ __forceinline__ FF ff_rsqrt(FF a) {  // 0 for a <= 0 (a singular precision)
-  if (!(a.h > 0.f)) return FF{a.h == a.h ? 0.f : a.h, 0.f};
-  const float y = rsqrtf(a.h);
-  const FF r = FF{1.f, 0.f} - a * ff_prod(y, y);
-  return ff_renorm(y, __fmul_rn(0.5f * y, r.h));
-}
-
 // The camera-plane records of a view (fmb_cam.cuh), one thread per Gaussian; the
 // threads of a pair exchange halves, so that each stores 64 consecutive bytes.  The
 // functions of R are those of the world-frame formulation (v = R^T c, o = -R^T t) for
@@ -230,6 +179,22 @@ __global__ void __launch_bounds__(128) prologue_cam_kernel(const __grid_constant
                          cam_flat_flags((P00 + P(1, 1) + P(2, 2)).h, m2.h, P00.h * S11.h * S22.h));
   w[14] = rho[0].h;
   w[15] = rho[1].h;
+  if (s.qrec != nullptr && real) {
+    // Q = B^-1 A by forward substitution (orthogonal; a row of zeros where P is singular)
+    const FF r2 = ff_rsqrt(S22);
+    float q[9];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const FF q0 = A[c] * r0, q1 = (A[3 + c] - B10 * q0) * r1, q2 = (A[6 + c] - B20 * q0 - B21 * q1) * r2;
+      q[c] = q0.h;
+      q[3 + c] = q1.h;
+      q[6 + c] = q2.h;
+    }
+    float4* d = s.qrec + kCamQFloat4 * (static_cast<long long>(V.rec_off) + i);
+    d[0] = make_float4(q[0], q[1], q[2], q[3]);
+    d[1] = make_float4(q[4], q[5], q[6], q[7]);
+    d[2] = make_float4(q[8], 0.f, 0.f, 0.f);
+  }
   const bool odd = (i & 1) != 0;
   float rv[8];
 #pragma unroll

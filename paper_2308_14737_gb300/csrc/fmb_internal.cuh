@@ -437,6 +437,9 @@ inline cudaError_t launch_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, 
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// B^-1 A of a (view, Gaussian), 9 floats and 3 of padding (fmb_backward.cu).
+constexpr int kCamQFloat4 = 3;
+
 struct Scene {
   const float* means;
   const float* chol;
@@ -444,6 +447,7 @@ struct Scene {
   const float* poses;
   const float* colors = nullptr;  // per-Gaussian RGB [G][3], or null
   float4* crec = nullptr;         // colour records (r, g, b, 0) per (view, Gaussian) in the workspace
+  float4* qrec = nullptr;         // camera-plane adjoint: kCamQFloat4 per (view, Gaussian) in the workspace
 };
 
 // Float arrays to clear (null entries skipped).

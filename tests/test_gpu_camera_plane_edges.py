@@ -176,3 +176,19 @@ def test_normals_of_thin_discs(K, seed, ratio):
         e = np.abs(plane_view(gpu["normal"], v, 3) - plane_view(ref["normal"], v, 3)).max(0) * nn
         e = e[ref["alpha"][v["pix_offset"]:][:len(e)] >= 1e-2]
         assert len(e) > 100 and np.sqrt(np.mean(e ** 2)) <= 2e-6
+
+
+@pytest.mark.parametrize("kind,ratio", [("disc", 30), ("disc", 100), ("disc", 300), ("needle", 30)])
+@pytest.mark.parametrize("K,seed", [(1, 0), (1, 1), (24, 0), (25, 1)])
+def test_gradients_of_thin_gaussians(kind, ratio, K, seed):
+    """With an upstream gradient of alpha alone the pairs' terms are well conditioned, so
+    what the axis ratio costs shows in L's and the poses' gradients: 1e-5 of the largest
+    entry, a tenth of the library's bound (sums of 32-bit terms carry about 1e-6)."""
+    s = _two_views(*_thin(K, ratio, kind, seed))
+    _, r, dev = gpu_forward(s, fmb.default_params(n_flow=1))
+    ga = np.random.default_rng(seed).standard_normal(s.n_pixels).astype(np.float32)
+    z = np.zeros(s.n_pixels, np.float32)
+    ups = dict(g_depth=z, g_alpha=ga, g_normal=np.tile(z, 3), g_flow=np.tile(z, 2))
+    g = gpu_backward(r, dev, ups)
+    compare_grads(g, oracle.backward_scene(s, *(ups[k] for k in ("g_depth", "g_alpha", "g_normal", "g_flow")), n_flow=1),
+                  rel=1e-5)
