@@ -192,3 +192,45 @@ def test_gradients_of_thin_gaussians(kind, ratio, K, seed):
     g = gpu_backward(r, dev, ups)
     compare_grads(g, oracle.backward_scene(s, *(ups[k] for k in ("g_depth", "g_alpha", "g_normal", "g_flow")), n_flow=1),
                   rel=1e-5)
+
+
+def _many_cancelling(zoom, W=401, H=331, K=2048):
+    mu, ch, lam = synth.random_gaussians(np.random.default_rng(0), K, "diag")
+    q = lambda x: float(np.float32(x))
+    view = dict(W=W, H=H, fx=q(zoom * W), fy=q(zoom * W), cx=W / 2.0, cy=H / 2.0, object=0, pose=0, flow_target=(-1, -1))
+    return synth.make_scene([(mu, ch, lam)], [view], [synth.look_at_pose((0.0, 0.0, -4.0))])
+
+
+@pytest.mark.parametrize("rpt", [0, 4])
+def test_scenes_whose_normals_all_nearly_cancel(rpt):
+    """With beta1 = 0.1 and a narrow field of view |N| is below 0.06 on most rays.  N carries
+    1e-6 per term's weight and direction, so err |N| stays below 5e-6, and the render takes
+    at most three times as long as without normals (1.5 times the operations; seven times
+    as long if every ray is summed again)."""
+    s = _many_cancelling(8.0)
+    assert s.n_pixels > WORLD_RAYS
+    ms = {}
+    for normals in (1, 0):
+        params = fmb.default_params(n_flow=0, want_normals=normals, fwd_rays_per_thread=rpt)
+        params.beta1, params.beta2 = 0.1, 0.3
+        gpu, r, dev = gpu_forward(s, params)
+        best = np.inf
+        for _ in range(5):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            r.forward(*dev)
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b))
+        ms[normals] = best
+        if normals:
+            b1, b2 = float(params.beta1), float(params.beta2)
+            pix = np.arange(0, s.n_pixels, 7)
+            v = s.views[0]
+            ref = oracle.render_view(s.means, s.chol, s.weights, s.poses[0], None,
+                                     (v["W"], v["H"], v["fx"], v["fy"], v["cx"], v["cy"]), pixels=pix, beta1=b1, beta2=b2)
+            nn = ref["saved"][:, 2]
+            assert np.mean(nn < 0.06) > 0.5
+            e = np.abs(plane_view(gpu["normal"], v, 3)[:, pix].T - ref["normal"]).max(1) * nn
+            assert np.all(e <= 5e-6), e.max()
+    assert ms[1] <= 3.0 * ms[0], ms
