@@ -9,8 +9,10 @@
 // registers: what leaves the window is blended at once -- transmittance, weight and
 // sums advance hit by hit, without scans, shuffles or a reduction -- and written back
 // as the new order.  A hit that would have to move by more than the window leaves it
-// out of order; the warp then walks again from the order just written, until every
-// ray's depths ascend.  Hits at exactly equal depth share the sum in front of their run
+// out of order; such rays are sorted by the whole warp, one after the other, and the
+// warp walks once more.  (Walking again from the order just written until every ray's
+// depths ascend took up to 20 times the warp-per-ray kernel's time on small images of
+// many Gaussians, 2.5 times on one 631x473 view at K = 256: 3.27 -> 0.65 ms.)  Hits at exactly equal depth share the sum in front of their run
 // (the indicator of Eq. 10 is strict).  Every pair's depth comes from pair_geom, as in
 // the warp-per-ray kernels, so that orders and ties are the same bits.
 //
@@ -63,11 +65,25 @@ int ac_walk_threads() { return kWalkThreads; }
 // 16 x 320x240 at K = 100: 384 / 768 / 1536 / 3000 columns per SM asked for 1081 / 932 /
 // 858 / 930 us (measured before the loop was split and unrolled); 631x473 at K = 61, one
 // round of columns of 2: 160 us against the warp kernel's 215.
-int ac_walk_run(long long total_rays, int sms) {
+// 0 also where the warp-per-ray kernel, which refines the previous pixel's order, is as
+// fast.  Hits change places in proportion to K / f from one pixel to the next (f: focal
+// length in pixels), and a sort costs about K log^2 K, so that the limit is on K^2 / f;
+// a launch (at most 64 views) needs 448 columns of 2 per SM.  Time of this kernel over
+// the warp kernel's, scenes of random / diagonal precisions:
+//   fewer columns: 210 per SM, K = 40 / 100 1.15 / 1.57, 0.83 / 1.55; 51 (800 views of 16x16) 1.2 to 2.1
+//   505 to 1580 columns, K^2 / f: K = 40 53 0.62 / 0.53, 125 0.90 / 0.81; K = 100 16 0.76 / 0.78, 78 1.00 /
+//     0.78, 100 0.97 / 0.80, 156 1.19 / 0.98; K = 160 80 0.90 / 0.66, 200 1.20 / 0.98; K = 256 105 1.39 / 0.99
+//   2590 and 4040 columns: K = 100 156 0.68 / 0.56; K = 160 250 0.69 / 0.60, 400 0.93 / 0.69; K = 256 64 0.96 /
+//     0.70, 205 1.33 / 1.01
+int ac_walk_run(long long total_rays, int launches, int maxK, float min_f, int sms) {
   const long long sm = std::max(sms, 1);
   int run = kWalkMaxRun;
   while (run > 2 && total_rays < 1536 * sm * run) run >>= 1;
-  return total_rays < 640 * sm * run ? 0 : run;
+  if (total_rays < 640 * sm * run) return 0;
+  const long long rays = total_rays / std::max(launches, 1);
+  if (rays < 448 * sm * 2) return 0;
+  const float limit = maxK <= 192 && rays >= 2000 * sm * 2 ? 400.f : (maxK <= 64 ? 128.f : 100.f);
+  return static_cast<float>(maxK) * static_cast<float>(maxK) > limit * min_f ? 0 : run;
 }
 
 template <bool NORMALS, int NFLOW, int M>
@@ -104,30 +120,10 @@ __global__ void __launch_bounds__(kWalkThreads) forward_ac_walk_kernel(const __g
     const int strip = u / W;
     const int p_first = strip * run * W + (u - strip * W);
 
-    // starting orders
-#pragma unroll 1
-    for (int src = 4; src < 32; src += 8) {
-      float vc[3], v[3], vl[3], pxy[2];
-      pixel_ray_dd(V, R, __shfl_sync(kFull, p_first, src), vc, v, vl, pxy);
-      unsigned long long key[M];
-#pragma unroll
-      for (int m = 0; m < M; ++m) {
-        const int e = (m << 5) | lane;
-        key[m] = kNoKey;
-        if (e < K) {
-          const AcPair q = ac_pair_eval<false>(srec + kAcRecStride * e, v, vl, k);
-          key[m] = (static_cast<unsigned long long>(order_bits(q.t)) << 32) | static_cast<unsigned>(e);
-        }
-      }
-      warp_bitonic_sort<M>(key, lane);
-      unsigned char* rows = orders + ((tid & ~31) + src - 4) * row_bytes;
-#pragma unroll
-      for (int m = 0; m < M; ++m)
-        if (lane * M + m < K)
-#pragma unroll
-          for (int r = 0; r < 8; ++r) rows[r * row_bytes + lane * M + m] = static_cast<unsigned char>(key[m]);
-    }
-    __syncwarp();
+    // Rays to sort before the next walk, and the rows of the warp that take a sorted order:
+    // first the starting orders.
+    unsigned todo = 0x10101010u;
+    int spread = 8;
 
 #pragma unroll 1
     for (int j = 0; j < run; ++j) {
@@ -137,8 +133,32 @@ __global__ void __launch_bounds__(kWalkThreads) forward_ac_walk_kernel(const __g
       float vc[3], v[3], vl[3], pxy[2];
       pixel_ray_dd(V, R, min(p, P - 1), vc, v, vl, pxy);
       float Sd = 0.f, Ws = 0.f, WT = 0.f, WN0 = 0.f, WN1 = 0.f, WN2 = 0.f, WC0 = 0.f, WC1 = 0.f, WC2 = 0.f;
-      // at most K walks sort any order (each moves every late hit forward by at least one)
-      for (int walk = 0; walk <= K; ++walk) {
+      for (int walk = 0; walk < 2; ++walk) {
+#pragma unroll 1
+        for (unsigned left = todo; left != 0; left &= left - 1) {
+          const int src = __ffs(left) - 1;
+          float sc[3], sv[3], sl[3], sxy[2];
+          pixel_ray_dd(V, R, __shfl_sync(kFull, min(p, P - 1), src), sc, sv, sl, sxy);
+          unsigned long long key[M];
+#pragma unroll
+          for (int m = 0; m < M; ++m) {
+            const int e = (m << 5) | lane;
+            key[m] = kNoKey;
+            if (e < K) {
+              const AcPair q = ac_pair_eval<false>(srec + kAcRecStride * e, sv, sl, k);
+              key[m] = (static_cast<unsigned long long>(order_bits(fminf(q.t, INFINITY))) << 32) | static_cast<unsigned>(e);
+            }
+          }
+          warp_bitonic_sort<M>(key, lane);
+          unsigned char* rows = orders + ((tid & ~31) + (src & ~(spread - 1))) * row_bytes;
+#pragma unroll
+          for (int m = 0; m < M; ++m)
+            if (lane * M + m < K)
+              for (int r = 0; r < spread; ++r) rows[r * row_bytes + lane * M + m] = static_cast<unsigned char>(key[m]);
+        }
+        todo = 0;
+        spread = 1;
+        __syncwarp();
         // the window: ascending depths, each with its Gaussian and ring slot (e | slot << 8)
         float wt[kWindow];
         int wi[kWindow];
@@ -210,7 +230,9 @@ __global__ void __launch_bounds__(kWalkThreads) forward_ac_walk_kernel(const __g
 #pragma unroll 2
         for (int i = kWindow; i < K; ++i) step(i, true, true);
         for (int i = max(K, kWindow); i < K + kWindow; ++i) step(i, false, true);
-        if (__all_sync(kFull, ascending)) break;
+        const unsigned late = __ballot_sync(kFull, !ascending);
+        if (late == 0 || walk > 0) break;  // the second walk is over sorted or ascending orders
+        todo = late;
       }
 
       if (in) {

@@ -413,10 +413,15 @@ Plan make_plan(const fmb_params* p, const long long* offs, int n_objects, int n_
     sms = 152;
   }
   if (ac) {
-    long long total = 0;
-    for (int i = 0; i < n_views; ++i) total += view_entries(views[i]);
-    pl.ac_run = fmb::ac_fwd_run(total, sms);
-    pl.ac_walk = fmb::ac_walk_run(total, sms);
+    int maxK = 1;
+    float min_f = INFINITY;
+    for (int i = 0; i < n_views; ++i) {
+      maxK = std::max(maxK, static_cast<int>(offs[views[i].object + 1] - offs[views[i].object]));
+      min_f = std::min({min_f, views[i].fx, views[i].fy});
+    }
+    const int launches = (n_views + fmb::kMaxBatchViews - 1) / fmb::kMaxBatchViews;
+    pl.ac_run = fmb::ac_fwd_run(entries, sms);
+    pl.ac_walk = fmb::ac_walk_run(entries, launches, maxK, min_f, sms);
     for (int i = 0; i < n_views; ++i)  // the entries of a ray batch are no columns of pixels
       if (views[i].rays != nullptr) pl.ac_walk = 0;
   }

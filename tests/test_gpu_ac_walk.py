@@ -76,3 +76,62 @@ def test_walk_agrees_with_warp_per_ray(K, views, W, H, opts, ties):
     gb = rb.backward(*x, g[0], g[1], gn, gf, colors=col, g_color=gc)
     for k in ga:
         assert (ga[k] - gb[k]).abs().max() <= 3e-5 * gb[k].abs().max(), k
+
+
+def _coarse(K, views, W, H, f, kind="cholesky"):
+    rng = np.random.default_rng(K)
+    obj = synth.random_gaussians(rng, K, kind)
+    pos = synth.sphere_positions(rng, min(views, 64))
+    vs = [dict(W=W, H=H, fx=float(f), fy=float(f), cx=W / 2.0, cy=H / 2.0, object=0, pose=i % len(pos),
+               flow_target=(-1, -1)) for i in range(views)]
+    return synth.make_scene([obj], vs, [synth.look_at_pose(p) for p in pos])
+
+
+def _both(s, params):
+    """The scene's renderer and one that lists the same pixels as ray batches."""
+    listed = [dict(v, rays=np.arange(v["W"] * v["H"])) for v in s.views]
+    return [fmb.Renderer(s.obj_offsets, vs, len(s.poses), params) for vs in (s.views, listed)]
+
+
+@pytest.mark.parametrize("K,views,W,H,f", [(256, 1, 631, 473, 60), (256, 16, 320, 240, 64), (200, 2, 801, 503, 100),
+                                           (128, 16, 128, 96, 16), (100, 64, 64, 48, 10), (9, 64, 64, 48, 1)])
+def test_orders_that_change_by_more_than_the_window(K, views, W, H, f):
+    """Wide fields of view, where the order changes by many places from one pixel to the
+    next: the warp-per-ray kernel's planes (1e-5, as above; of the scene's unit where hits in
+    front of and behind the camera cancel in the depth) and depth orders."""
+    s = _coarse(K, views, W, H, f)
+    assert s.n_pixels >= 640 * 2 * 152
+    x = dev_scene(s)
+    r, rb = _both(s, fmb.default_params(variant=1, want_normals=0, n_flow=0, keep_order=1))
+    a = {k: t.clone() for k, t in r.forward(*x).items() if t is not None}
+    b = rb.forward(*x)
+    seen = b["alpha"] >= 1e-2
+    assert (a["alpha"] - b["alpha"]).abs().max() <= 1e-5
+    assert ((a["depth"] - b["depth"]).abs() / b["depth"].abs().clamp(min=1.0))[seen].max() <= 1e-5
+    torch.manual_seed(0)
+    g = [torch.randn(s.n_pixels, device="cuda") * seen, torch.randn(s.n_pixels, device="cuda") * seen]
+    ga, gb = r.backward(*x, *g, None, None), rb.backward(*x, *g, None, None)
+    for k in ga:
+        assert (ga[k] - gb[k]).abs().max() <= 3e-5 * gb[k].abs().max(), k
+
+
+@pytest.mark.parametrize("K,views,W,H,f", [(256, 1, 631, 473, 631), (256, 16, 128, 96, 128), (100, 250, 32, 32, 32),
+                                           (256, 100, 64, 48, 64), (100, 800, 16, 16, 16), (40, 3200, 8, 8, 2)])
+@pytest.mark.parametrize("kind", ["cholesky", "diag"])
+def test_no_slower_than_warp_per_ray(K, views, W, H, f, kind):
+    """Whatever the planner takes for whole images is not slower than the warp-per-ray
+    kernel that ray batches take (with a quarter to spare for the clock)."""
+    s = _coarse(K, views, W, H, f, kind)
+    x = dev_scene(s)
+    ms = []
+    for r in _both(s, fmb.default_params(variant=1, want_normals=0, n_flow=0)):
+        best = np.inf
+        for _ in range(5):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            r.forward(*x)
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b))
+        ms.append(best)
+    assert ms[0] <= 1.25 * ms[1], ms
