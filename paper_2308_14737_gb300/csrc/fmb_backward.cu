@@ -789,10 +789,15 @@ __device__ __forceinline__ float warp_sum_fixed(float x) {
 
 // Gaussian gradients: warp w handles (Gaussian g, component comp), w = g * nc + comp
 // (nc = 10, or 13 with colours: means 3, chol 6, weight 1, colour 3).
+__device__ __forceinline__ float* gauss_grad(const BwdOut& out, long long g, int comp) {
+  if (comp < 3) return out.gmeans + 3 * g + comp;
+  if (comp < 9) return out.gchol + 6 * g + comp - 3;
+  if (comp == 9) return out.gweights + g;
+  return out.gcolors + 3 * g + comp - 10;
+}
+
 template <class B>
-__global__ void reduce_gauss_kernel(const __grid_constant__ B batch, const float* __restrict__ partials,
-                                    float* gmeans, float* gchol, float* gweights, float* gcolors, long long n_gauss,
-                                    int nc, int slots, bool spread) {
+__global__ void reduce_gauss_kernel(const __grid_constant__ B batch, BwdOut out, long long n_gauss, int nc) {
   pdl_enter();
   const long long w = (blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -801,75 +806,98 @@ __global__ void reduce_gauss_kernel(const __grid_constant__ B batch, const float
   const int comp = static_cast<int>(w - g * nc);
   float acc = 0.f;
   bool hit = false;
-  // spread (slots, all views of one object): groups of kAccSlots lanes take one view each.
-  // 16 x 320x240 at K = 100: 659 -> 650 us for render and adjoint; with 24 objects, where a
-  // Gaussian is in few of the views, 9106 -> 9295 us (the groups read the table apart), so not there
-  const int vstep = spread ? 32 / kAccSlots : 1;
-  const int l0 = spread ? lane % kAccSlots : lane, lstep = spread ? kAccSlots : 32;
-  for (int v = spread ? lane / kAccSlots : 0; v < batch.n_views; v += vstep) {
+  for (int v = 0; v < batch.n_views; ++v) {
     const DevView& V = batch.v[v];
     if (g < V.gauss_off || g >= V.gauss_off + V.K) continue;
     hit = true;
     const int gi = static_cast<int>(g - V.gauss_off);
     const int gbk = gi / V.GB, gl = gi - gbk * V.GB;
-    const int n = slots > 0 ? min(slots, V.n_tiles) : V.n_tiles;
-    for (int t = l0; t < n; t += lstep)
-      acc += partials[V.part_off + static_cast<long long>(t * V.n_gblocks + gbk) * V.slot_floats + nc * gl + comp];
+    for (int t = lane; t < V.n_tiles; t += 32)
+      acc += out.partials[V.part_off + static_cast<long long>(t * V.n_gblocks + gbk) * V.slot_floats + nc * gl + comp];
   }
   acc = warp_sum_fixed(acc);
-  hit = __any_sync(0xffffffffu, hit);
-  if (!hit || lane != 0) return;
-  if (comp < 3)
-    gmeans[3 * g + comp] += acc;
-  else if (comp < 9)
-    gchol[6 * g + comp - 3] += acc;
-  else if (comp == 9)
-    gweights[g] += acc;
-  else
-    gcolors[3 * g + comp - 10] += acc;
+  if (hit && lane == 0) *gauss_grad(out, g, comp) += acc;
 }
 
 // Pose gradients: warp w handles (pose p, component comp), w = p * 12 + comp.
 template <class B>
-__global__ void reduce_pose_kernel(const __grid_constant__ B batch, const float* __restrict__ partials,
-                                   float* gposes, int n_poses, int n_flow, int nc, int slots, bool spread) {
+__global__ void reduce_pose_kernel(const __grid_constant__ B batch, BwdOut out, int n_poses, int n_flow, int nc) {
   pdl_enter();
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (w >= n_poses * 12) return;
   const int p = w / 12, comp = w % 12;
   float acc = 0.f;
-  const int vstep = spread ? 32 / kAccSlots : 1;
-  const int l0 = spread ? lane % kAccSlots : lane, lstep = spread ? kAccSlots : 32;
-  for (int v = spread ? lane / kAccSlots : 0; v < batch.n_views; v += vstep) {
+  for (int v = 0; v < batch.n_views; ++v) {
     const DevView& V = batch.v[v];
     for (int j = -1; j < n_flow; ++j) {
       const int pidx = j < 0 ? V.pose : (j == 0 ? V.tgt0 : V.tgt1);
       if (pidx != p) continue;
       const int part = 12 * (j + 1) + comp;
-      const int nslots = (slots > 0 ? min(slots, V.n_tiles) : V.n_tiles) * V.n_gblocks;
-      for (int sl = l0; sl < nslots; sl += lstep)
-        acc += partials[V.part_off + static_cast<long long>(sl) * V.slot_floats + nc * V.GB + part];
+      const int nslots = V.n_tiles * V.n_gblocks;
+      for (int sl = lane; sl < nslots; sl += 32)
+        acc += out.partials[V.part_off + static_cast<long long>(sl) * V.slot_floats + nc * V.GB + part];
     }
   }
   acc = warp_sum_fixed(acc);
-  if (lane == 0) gposes[12 * static_cast<long long>(p) + comp] += acc;
+  if (lane == 0) out.gposes[12 * static_cast<long long>(p) + comp] += acc;
+}
+
+// The slots of atomic mode, view by view: a thread adds the (at most kAccSlots) slots of
+// one value of one view and adds that to the gradient, so the work follows what was
+// rendered.  (A warp per value that looks for it in every view, as above, took 57 ms
+// after 2.0 ms of adjoint for 256 objects of 1024 Gaussians, one 64x64 view each.)
+template <class B>
+__global__ void __launch_bounds__(256) add_slots_gauss_kernel(const __grid_constant__ B batch, BwdOut out, int nc) {
+  pdl_enter();
+  const DevView& V = batch.v[blockIdx.y];
+  const long long e = blockIdx.x * 256ll + threadIdx.x;
+  if (e >= static_cast<long long>(V.K) * nc) return;
+  const int gi = static_cast<int>(e / nc), comp = static_cast<int>(e - static_cast<long long>(gi) * nc);
+  const int gbk = gi / V.GB;
+  const float* src = out.partials + V.part_off + static_cast<long long>(gbk) * V.slot_floats + nc * (gi - gbk * V.GB) + comp;
+  const long long step = static_cast<long long>(V.n_gblocks) * V.slot_floats;
+  const int n = min(out.slots, V.n_tiles);
+  float acc = 0.f;
+  for (int t = 0; t < n; ++t) acc += src[t * step];
+  atomicAdd(gauss_grad(out, V.gauss_off + gi, comp), acc);
+}
+// A warp per value of a view's pose sums.
+template <class B>
+__global__ void __launch_bounds__(384) add_slots_pose_kernel(const __grid_constant__ B batch, BwdOut out, int n_flow, int nc) {
+  pdl_enter();
+  const DevView& V = batch.v[blockIdx.x];
+  const int lane = threadIdx.x & 31, comp = threadIdx.x >> 5;
+  const int nslots = min(out.slots, V.n_tiles) * V.n_gblocks;
+  for (int j = -1; j < n_flow; ++j) {
+    const int pidx = j < 0 ? V.pose : (j == 0 ? V.tgt0 : V.tgt1);
+    if (pidx < 0) continue;
+    const float* src = out.partials + V.part_off + nc * V.GB + 12 * (j + 1) + comp;
+    float acc = 0.f;
+    for (int sl = lane; sl < nslots; sl += 32) acc += src[static_cast<long long>(sl) * V.slot_floats];
+    acc = warp_sum_fixed(acc);
+    if (lane == 0) atomicAdd(out.gposes + 12 * static_cast<long long>(pidx) + comp, acc);
+  }
 }
 
 template <class B>
 static cudaError_t launch_backward_reduce_t(const B& b, int n_flow, long long n_gauss, int n_poses,
                                             const BwdOut& out, cudaStream_t st) {
   const int nc = out.gcolors != nullptr ? 13 : 10;
-  bool spread = out.slots > 0;
-  for (int i = 0; i < b.n_views; ++i) spread = spread && b.v[i].gauss_off == b.v[0].gauss_off;
+  if (out.slots > 0) {
+    long long values = 0;
+    for (int i = 0; i < b.n_views; ++i) values = std::max(values, static_cast<long long>(b.v[i].K) * nc);
+    const dim3 grid(static_cast<unsigned>((values + 255) / 256), static_cast<unsigned>(b.n_views));
+    const cudaError_t e = launch_kernel(add_slots_gauss_kernel<B>, grid, dim3(256), 0, st, 1, b, out, nc);
+    if (e != cudaSuccess || out.gposes == nullptr) return e;
+    return launch_kernel(add_slots_pose_kernel<B>, dim3(b.n_views), dim3(384), 0, st, 1, b, out, n_flow, nc);
+  }
   const long long warps = n_gauss * nc;
   const dim3 grid(static_cast<unsigned>((warps * 32 + 255) / 256));
-  const float* partials = out.partials;
-  cudaError_t e = launch_kernel(reduce_gauss_kernel<B>, grid, dim3(256), 0, st, 1, b, partials, out.gmeans,
-                                out.gchol, out.gweights, out.gcolors, n_gauss, nc, out.slots, spread);
+  const cudaError_t e = launch_kernel(reduce_gauss_kernel<B>, grid, dim3(256), 0, st, 1, b, out, n_gauss, nc);
   if (e != cudaSuccess || out.gposes == nullptr) return e;
-  return launch_kernel(reduce_pose_kernel<B>, dim3((n_poses * 12 * 32 + 255) / 256), dim3(256), 0, st, 1, b,
-                       partials, out.gposes, n_poses, n_flow, nc, out.slots, spread);
+  return launch_kernel(reduce_pose_kernel<B>, dim3((n_poses * 12 * 32 + 255) / 256), dim3(256), 0, st, 1, b, out,
+                       n_poses, n_flow, nc);
 }
 cudaError_t launch_backward_reduce(const Batch& b, int n_flow, long long n_gauss, int n_poses, const BwdOut& out,
                                    cudaStream_t st) {

@@ -514,13 +514,11 @@ struct FwdOut {
 cudaError_t launch_zero(const ZeroJob& job, cudaStream_t st);
 
 // Camera-plane adjoint, atomic mode: the CTAs add their sums into this many slots per
-// view and Gaussian block of the workspace, and the deterministic mode's second stage
-// adds the slots.  Added straight into the gradients, 8 views of 1024x768 at K = 4096
+// view and Gaussian block of the workspace, and a second stage adds the slots.  Added straight into the gradients, 8 views of 1024x768 at K = 4096
 // make 12 288 fp32 additions per Gaussian value and more than 24 000 per pose value,
 // whose rounding (about sqrt(n) 2^-25) was most of the gradients' error: largest error
 // against 64 bits 4.2e-6 to 6.8e-6 by seed, 2.4e-6 with the slots.
 constexpr int kAccSlots = 8;
-static_assert(32 % kAccSlots == 0, "the reductions give a view kAccSlots lanes");
 
 struct BwdOut {
   float* gmeans;

@@ -234,3 +234,64 @@ def test_scenes_whose_normals_all_nearly_cancel(rpt):
             e = np.abs(plane_view(gpu["normal"], v, 3)[:, pix].T - ref["normal"]).max(1) * nn
             assert np.all(e <= 5e-6), e.max()
     assert ms[1] <= 3.0 * ms[0], ms
+
+
+def _many_objects(n_obj, K, n_views, side, shown):
+    """n_views square views, view i of object i mod shown of n_obj equal ones."""
+    rng = np.random.default_rng(4)
+    obj = synth.random_gaussians(rng, K)
+    views = [dict(W=side, H=side, fx=float(side), fy=float(side), cx=side / 2.0, cy=side / 2.0, object=(7 * i) % shown,
+                  pose=i, flow_target=((i + 1) % n_views, i - 1)) for i in range(n_views)]
+    return synth.make_scene([obj] * n_obj, views, [synth.look_at_pose(p) for p in synth.sphere_positions(rng, n_views)])
+
+
+@pytest.mark.parametrize("n_obj,K,n_views,side,shown,colors", [
+    (5, 37, 11, 129, 3, 0), (40, 21, 70, 50, 33, 0), (300, 9, 300, 29, 299, 1), (3, 515, 5, 201, 2, 0)])
+def test_slots_of_several_objects(n_obj, K, n_views, side, shown, colors):
+    """Gradients of several objects (one to five launches' views, objects that no view
+    shows) through the slots against the deterministic mode: the same terms in another
+    order, 3e-5 of the largest entry."""
+    s = _many_objects(n_obj, K, n_views, side, shown)
+    assert s.n_pixels > WORLD_RAYS
+    x = dev_scene(s)
+    torch.manual_seed(n_obj)
+    P = s.n_pixels
+    col = torch.rand(n_obj * K, 3, device="cuda") if colors else None
+    got, ups = [], None
+    for det in (0, 1):
+        r = fmb.Renderer(s.obj_offsets, s.views, len(s.poses), fmb.default_params(n_flow=2, colors=colors, deterministic=det))
+        out = r.forward(*x, colors=col)
+        if ups is None:
+            on = out["alpha"] >= 1e-2
+            planes = lambda n: torch.cat([torch.randn(n, side * side, device="cuda") *
+                                          on[i * side * side:(i + 1) * side * side] for i in range(n_views)]).reshape(-1)
+            nn = out["saved"].view(n_views, 3, -1)[:, 2:].expand(n_views, 3, -1).reshape(-1)
+            ups = [planes(1), torch.randn(P, device="cuda"), planes(3) * (nn >= 0.05), 0.01 * planes(4)]
+            gc = planes(3) if colors else None
+        got.append(r.backward(*x, *ups, colors=col, g_color=gc))
+    for k, t in got[1].items():
+        assert (got[0][k].double() - t.double()).abs().max() <= 3e-5 * t.abs().max(), k
+    for k in ("means", "chol", "weights"):
+        assert not got[0][k].view(n_obj, -1)[shown:].any()
+
+
+@pytest.mark.parametrize("n_obj,K,n_views,side,shown", [(256, 1024, 256, 64, 256), (4000, 1000, 64, 112, 64)])
+def test_the_adjoint_of_many_objects_follows_what_is_rendered(n_obj, K, n_views, side, shown):
+    """The time of the adjoint does not depend on how many objects the rays are spread
+    over: twice one object's time at most, plus 1 ms for clearing the other gradients."""
+    ms = []
+    for obj, sh in ((n_obj, shown), (1, 1)):
+        s = _many_objects(obj, K, n_views, side, sh)
+        x = dev_scene(s)
+        r = fmb.Renderer(s.obj_offsets, s.views, len(s.poses), fmb.default_params(n_flow=0, want_normals=0))
+        on = (r.forward(*x)["alpha"] >= 1e-2).float()
+        best = np.inf
+        for _ in range(4):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            r.backward(*x, on, on, None, None)
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b))
+        ms.append(best)
+    assert ms[0] <= 2.0 * ms[1] + 1.0, ms
