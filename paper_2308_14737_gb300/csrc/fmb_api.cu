@@ -389,11 +389,17 @@ Plan make_plan(const fmb_params* p, const long long* offs, int n_objects, int n_
   Plan pl;
   const long long entries = total_entries(views, n_views);
   pl.world = p->variant == 0 && (p->store_pairs || entries <= kWorldRays);
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();  // no device (a host-only size query): plan for 152 SMs
+    sms = 152;
+  }
   // Four rays per thread where that still leaves the camera-plane forward (3 resident
   // CTAs per SM) four rounds of CTAs: 16 x 320x240 at K = 100 186 against 190 us with
   // two, 20 x 640x480 at K = 256 without normals 1.44 against 1.52 ms, one 1024x768 view
   // at K = 4096 4.47 against 4.54 ms; but 1023x767 at K = 333 363 against 358 us.
-  const bool many = p->variant == 0 && !pl.world && !p->colors && entries >= 6144ll * 152;
+  const bool many = p->variant == 0 && !pl.world && !p->colors && entries >= 6144ll * std::max(sms, 1);
   pl.rpt = p->fwd_rays_per_thread > 0 ? p->fwd_rays_per_thread : (many ? 4 : kDefaultRpt);
   pl.bwd_threads = p->bwd_threads > 0
                        ? p->bwd_threads
@@ -406,12 +412,6 @@ Plan make_plan(const fmb_params* p, const long long* offs, int n_objects, int n_
   pl.ray_tile = p->bwd_ray_tile > 0 ? p->bwd_ray_tile : (pl.world ? 3 : 4) * pl.bwd_threads;
   pl.n_gauss = offs[n_objects];
   const bool ac = p->variant == 1;
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();  // no device (a host-only size query): plan for 152 SMs
-    sms = 152;
-  }
   if (ac) {
     int maxK = 1;
     float min_f = INFINITY;
