@@ -13,8 +13,8 @@ steps, outside the timed events.
                     [--workload largek|orbit|single|ragged|recon|minibatch]
                     [--configs all|none]
 
-At N = 1 the same JSON line carries, under "configs", one record for each of the
-other configurations, measured the same way in the same run: a single 64x64 view
+At N = 1 the record carries, under "configs", one record for each of the other
+configurations, measured the same way in the same run: a single 64x64 view
 with K = 40 (depth + alpha, Gaussian gradients); the 16-view 320x240 orbit with
 K = 100 (all planes, flow, pose gradients); the ragged batch of 64 objects (K from
 20 to 400, square images of side 64..512, 4 views each); and the reconstruction
@@ -30,7 +30,8 @@ The batched arm's tiles come from the autotuner, run before the timed region; se
 FMB_AUTOTUNE_CACHE to a file to reuse a previous run's choice (e.g. when
 profiling, so the profiled run launches no tuning candidates).
 
-Prints one JSON line.  Under torchrun (N > 1) every rank renders its own replica
+Prints one JSON line (``result_line``: under 2 KB, with the rate and time of each
+further configuration); the whole record goes to stderr as one line.  Under torchrun (N > 1) every rank renders its own replica
 of the headline batch (weak scaling) and rank 0 prints the aggregate.
 """
 
@@ -544,6 +545,22 @@ def measure_workload(args, name, steps, warmup, dev, ws=1, extras=True, cpu=True
     return rec
 
 
+def result_line(line):
+    """The result line: the whole record without its explanations and with one rate and
+    time per further configuration, so that it stays under 2 KB whatever was measured (a
+    reader that keeps the last few KB of the output gets all of it)."""
+    out = {k: v for k, v in line.items() if k in (
+        "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+        "vs_baseline", "dtype", "data", "config", "fwd_ms", "bwd_ms", "batched_over_plain", "gpu_launches")}
+    pick = lambda d, keys: {k: d[k] for k in keys if k in d}
+    out["roofline"] = pick(line["roofline"], ("bound", "achieved", "peak", "frac", "step_frac"))
+    out["clocks"] = pick(line["clocks"], ("sm_mhz", "sm_max_mhz", "reasons"))
+    out["e2e"] = pick(line["e2e"], ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_step"))
+    if "configs" in line:
+        out["configs"] = {name: pick(rec, ("value", "ms_per_step")) for name, rec in line["configs"].items()}
+    return out
+
+
 def timed_call(fn, steps, dev, pairs, what):
     """A call timed alone after three warm-up calls: mean of max(steps / 4, 3)."""
     import torch
@@ -624,7 +641,8 @@ def run_gpu(args):
             line[k] = head[k]
     if subs:
         line["configs"] = subs
-    print(json.dumps(line), flush=True)
+    print(json.dumps(line), file=sys.stderr, flush=True)  # everything that was measured
+    print(json.dumps(result_line(line)), flush=True)
     if ws > 1:
         torch.distributed.barrier()
         torch.distributed.destroy_process_group()

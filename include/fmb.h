@@ -77,7 +77,9 @@ typedef struct {
                         holds W = sum of the weights instead of the log2 normaliser) */
   int want_normals;  /* 1: compute the blended normal plane (Eq. 17) and its adjoint */
   int n_flow;        /* flow slots per view, 0..2 (Sec. 5: forward i+1 and backward i-1) */
-  int deterministic; /* backward: 1 = fixed-order two-stage reduction, 0 = fp32 atomics */
+  int deterministic; /* backward: 1 = fixed-order two-stage reduction, 0 = fp32 atomics (into
+                        the gradients, or for calls of more than 131 072 rays into up to
+                        eight partial sums per view in the workspace, then added up) */
   int use_persistent;/* 1: persistent launch (one grid of resident CTAs popping (view, tile)
                         work items, most expensive first, from a counter in the workspace);
                         0: one CTA per work item */
@@ -211,7 +213,9 @@ fmb_status fmb_render_forward(const fmb_params* params, int n_objects, const lon
  * [n_poses][12] (d/dR as a free 3x3 matrix, row-major, then d/dt; NULL = pose
  * gradients not computed).
  * deterministic = 1 gives bitwise-reproducible results (fixed-order two-stage
- * reduction through the workspace); 0 uses fp32 atomics.
+ * reduction through the workspace); 0 uses fp32 atomics (of two-parameter calls of more
+ * than 131 072 rays into up to eight partial sums per view in the workspace, which a
+ * second stage adds up; smaller calls and variant 1 straight into the gradients).
  */
 fmb_status fmb_render_backward(const fmb_params* params, int n_objects, const long long* h_obj_offsets,
                                const float* means, const float* chol, const float* weights, const float* colors,
@@ -230,11 +234,11 @@ fmb_status fmb_render_backward(const fmb_params* params, int n_objects, const lo
  * deployment variant of the same forward render, with the same arguments,
  * layouts and results minus `workspace`/`workspace_bytes`.
  *
- * Its scratch is one fixed 1 MiB array in the library (held on every device that
- * loads the library until the process exits): a batch needs 256 + 64 x (sum over
- * views of the view's Gaussian count) bytes (plus 16 more per view and Gaussian
- * with colours, each region rounded up to 256), and a larger batch is rejected with
- * FMB_ERR_WORKSPACE.  Nothing is allocated.  The first call on each device looks up
+ * Its scratch is one fixed 2 MiB array in the library (held on every device that
+ * loads the library until the process exits).  A batch may need 1 MiB, counted as 256 +
+ * 64 x (sum over views of the view's Gaussian count) bytes (plus 16 more per view and
+ * Gaussian with colours, each region rounded up to 256); the rest holds the padding of
+ * odd counts.  A larger batch is rejected with FMB_ERR_WORKSPACE.  Nothing is allocated.  The first call on each device looks up
  * the array's device address (cudaGetSymbolAddress); make that first call before
  * any stream capture.  All calls share the array: calls whose GPU work overlaps
  * (different streams or host threads) race on it.  The device address is cached
@@ -323,8 +327,9 @@ int fmb_forward_ksplit(const fmb_params* params, int n_objects, const long long*
  * paper has no counterpart: this reports a launch decision of this
  * implementation (the batch is split into launches of at most a fixed number of
  * views: 64, or 256 for a two-parameter forward or backward of more than 64
- * views; a Gaussian-split forward adds a merge; deterministic mode adds the
- * second-stage reductions). */
+ * views; a Gaussian-split forward adds a merge; a backward that adds partial sums up
+ * (deterministic mode, and two-parameter calls of more than 131 072 rays) adds one
+ * launch, or two with pose gradients, per batch). */
 int fmb_launch_count(const fmb_params* params, int n_objects, const long long* h_obj_offsets, int n_views,
                      const fmb_view* h_views, int pass, int want_pose);
 

@@ -44,10 +44,13 @@ constexpr int kDefaultRpt = 2;
 // of the operations.  Both have the same error against FP64 on average, but not the same
 // rounding: over 12 scenes the ratio of their gradient errors spreads by a factor of
 // 1.3-1.7 for one view of 9 000 to 120 000 rays, where single rays show in the sums, and
-// by 1.2 from 300 000 rays on.  Small calls have little to gain: they are bound by
-// latency and launches (64x64 view at K = 40, forward and backward replayed: 41.5 us
-// world, 38.1 camera; 50 000-ray minibatch at K = 256, eager calls: 167 and 166 us),
-// while 150 000 rays at K = 100-4096 already gain 1.2-1.35x.
+// by 1.2 from 300 000 rays on.  So a scene's result depends, within that rounding, on
+// whether its views come in one call or several.  Small calls of few Gaussians have
+// little to gain: they are bound by latency and launches (64x64 view at K = 40, forward
+// and backward replayed: 41.5 us world, 38.1 camera; 50 000-ray minibatch at K = 256, eager
+// calls: 167 and 166 us).  From 150 000 rays on the gain is 1.2-1.35x at K = 100-4096.  The
+// rule looks at rays alone: calls of few rays and many Gaussians are bound by the FP32
+// pipe too, and stay on the slower form.
 constexpr long long kWorldRays = 131072;
 constexpr int kMaxGaussPerCta = 256;
 constexpr long long kMaxK = 1 << 22;

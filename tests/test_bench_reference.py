@@ -49,3 +49,32 @@ def test_profile_gate_follows_sources_and_compile_flags(monkeypatch):
     monkeypatch.setitem(build.EXTRA_FLAGS, "fmb_backward.cu", [])
     assert bench.csrc_sha256() != sha
     assert bench.profiled_traffic(tiles) is None
+
+
+def test_result_line_stays_short():
+    """The GPU arm's result line keeps every key of the contract and stays under 2 KB, however
+    long the record of explanations and further configurations is."""
+    sys.path.insert(0, ROOT)
+    import bench
+
+    s, _ = bench.scene_and_inputs(workload=bench.DEFAULT_WORKLOAD)
+    x, text = 123456789012.34567, "explanation " * 200
+    config = dict(bench.workload_config(s, bench.WORKLOADS[bench.DEFAULT_WORKLOAD]), parallelism="single GPU")
+    rec = {"value": x, "ms_per_step": x, "roofline": {"frac": x, "what": text}, "note": text}
+    full = {"metric": bench.METRIC, "value": x, "unit": "pairs/s", "n_gpus": 1, "steps": 20, "warmup": 5, "ms_per_step": x,
+            "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32",
+            "data": "synthetic (seeded; stands in for the paper's CO3D sequences)", "config": config, "launch": {"w": text},
+            "plain": rec, "batched_over_plain": x, "fwd_ms": x, "bwd_ms": x, "frames_per_s": x, "paper_context": text,
+            "roofline": {"bound": "alu", "achieved": x, "peak": x, "frac": x, "step_frac": x, "forward": rec},
+            "clocks": {"sm_mhz": x, "sm_max_mhz": x, "reasons": ["sw_power_cap"], "samples": 9}, "gpu_launches": 80,
+            "e2e": {"value": x, "unit": "pairs/s", "h2d_bytes_per_step": 10 ** 9, "d2h_bytes_per_step": 10 ** 9,
+                    "ms_per_step": x, "what": text}, "cpu_baseline": rec, "recon_step": rec,
+            "configs": {name: rec for name in bench.SUB_CONFIGS}}
+    line = json.dumps(bench.result_line(full))
+    assert len(line) < 2048, len(line)
+    d = json.loads(line)
+    for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+              "vs_baseline", "dtype", "data", "config", "clocks", "gpu_launches", "e2e"):
+        assert k in d, k
+    assert d["config"] == json.loads(json.dumps(config))
+    assert set(d["e2e"]) >= {"value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"}
