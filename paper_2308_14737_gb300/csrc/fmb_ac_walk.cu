@@ -19,10 +19,10 @@
 // The first pixel of a column starts from a warp's bitonic sort of a ray at most four
 // pixels away (four sorts per warp).
 //
-// Bound by its instructions (78 % of the issue rate, the compares and selects of the
-// window half of them; 500 warp instructions per ray against the warp-per-ray kernel's
-// 1225).  Orbit of 16 views 320x240, K = 100, depth, alpha and flow: 1.340 -> 0.699 ms;
-// with normals 1.452 -> 0.853 ms.
+// Bound by its instructions (76 % of the issue rate, the compares and selects of the
+// window half of them; 562 warp instructions per ray with normals against the warp-per-ray
+// kernel's 1225).  Orbit of 16 views 320x240, K = 100, depth, alpha and flow: 1.340 -> 0.699
+// ms; with normals 1.452 -> 0.848 ms.
 #include <algorithm>
 
 #include "fmb_ac.cuh"
