@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kWalkThreads) forward_ac_walk_kernel(const __g
 #pragma unroll 2
         for (int i = kWindow; i < K; ++i) step(i, true, true);
         for (int i = max(K, kWindow); i < K + kWindow; ++i) step(i, false, true);
-        const unsigned late = __ballot_sync(kFull, !ascending);
+        const unsigned late = __ballot_sync(kFull, in && !ascending);
         if (late == 0 || walk > 0) break;  // the second walk is over sorted or ascending orders
         todo = late;
       }
