@@ -883,7 +883,11 @@ fmb_status fmb_loss_attribution(const fmb_params* params, int n_objects, const l
     bool first = true;  // the first batch's prologue clears the attribution output
     if (params->variant == 0) {
       // two-parameter model: the backward's blocking (two Gaussians per thread)
-      const int T = pl.bwd_threads;
+      // by the world-frame form's cost, which the attribution kernel shares (16 views of
+      // 320x240 at K = 150: 160 threads 320 us, the 128 of the camera-plane adjoint 336)
+      const int T = params->bwd_threads > 0 ? params->bwd_threads
+                                            : choose_bwd_threads(h_views, n_views, h_obj_offsets, params->bwd_gblocks,
+                                                                 params->store_pairs != 0, true);
       const int tile = fmb::attribution2_ray_tile(T);
       for (fmb::Batch b : pl.fwd) {
         for (int i = 0; i < b.n_views; ++i) {
