@@ -410,9 +410,14 @@ Plan make_plan(const fmb_params* p, const long long* offs, int n_objects, int n_
                                             pl.world || p->variant == 1);
   // default ray tile: three rays per thread in the per-ray phase (balanced, and long
   // enough to amortise the per-CTA reductions); four in the camera-plane form, whose ray
-  // records are smaller (orbit adjoint 455 -> 449 us, K = 256 without normals 3.03 ->
-  // 2.98 ms for 20 views, one view at K = 4096 10.17 -> 10.20 ms)
-  pl.ray_tile = p->bwd_ray_tile > 0 ? p->bwd_ray_tile : (pl.world ? 3 : 4) * pl.bwd_threads;
+  // records are smaller, where that leaves every SM 15 CTAs (orbit adjoint 455 -> 449 us,
+  // K = 256 without normals 3.03 -> 2.98 ms for 20 views, one view at K = 4096 10.17 -> 10.20
+  // ms).  With fewer CTAs the longer tiles leave SMs idle: 150 000 rays over 100 views at
+  // K = 256 without normals 141 us with three, 178 with four (147 in the world-frame form),
+  // 200 views of 32x32 134 and 184 (149), one 500x400 view at K = 160 141 and 181 (170), one
+  // 1024x768 view at K = 160 458 and 492.
+  const bool four = !pl.world && entries >= 15ll * std::max(sms, 1) * 4 * pl.bwd_threads;
+  pl.ray_tile = p->bwd_ray_tile > 0 ? p->bwd_ray_tile : (four ? 4 : 3) * pl.bwd_threads;
   pl.n_gauss = offs[n_objects];
   const bool ac = p->variant == 1;
   if (ac) {

@@ -295,3 +295,33 @@ def test_the_adjoint_of_many_objects_follows_what_is_rendered(n_obj, K, n_views,
             best = min(best, a.elapsed_time(b))
         ms.append(best)
     assert ms[0] <= 2.0 * ms[1] + 1.0, ms
+
+
+@pytest.mark.parametrize("n_views,side,rays,K,normals", [(100, 200, 150000, 256, 0), (200, 32, 0, 256, 0),
+                                                         (1, 448, 0, 160, 1), (16, 277, 0, 100, 1)])
+def test_default_ray_tile_suits_the_call(n_views, side, rays, K, normals):
+    """The planner's ray tile is not slower than three or four rays per thread asked for,
+    whichever is better (with an eighth to spare for the clock): long tiles leave SMs idle
+    in calls of a few hundred thousand rays."""
+    s = _many_objects(1, K, n_views, side, 1)
+    if rays:
+        s = synth.ray_batch(s, rays, 0)
+    assert s.n_pixels > WORLD_RAYS
+    x = dev_scene(s)
+    P, ms = s.n_pixels, {}
+    for tile in (0, 384, 512):
+        params = fmb.default_params(n_flow=0, want_normals=normals, bwd_threads=128, bwd_ray_tile=tile)
+        r = fmb.Renderer(s.obj_offsets, s.views, len(s.poses), params)
+        up = (r.forward(*x)["alpha"] >= 1e-2).float()
+        gn = torch.zeros(3 * P, device="cuda") if normals else None
+        best = np.inf
+        for _ in range(4):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            for _ in range(20):
+                r.backward(*x, up, up, gn, None, want_pose=False)
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b))
+        ms[tile] = best
+    assert ms[0] <= 1.125 * min(ms[384], ms[512]), ms
