@@ -148,7 +148,13 @@ struct CamGeom2 {
   f2 dx, dy, a0, a1, ninv, tau, t, u0, u1, nx;  // ninv = -1 / a.a;  nx = -log2(delta)
 };
 __device__ __forceinline__ f2 rcp_neg_2(f2 a) { return pk(rcp_approx(-lo(a)), rcp_approx(-hi(a))); }
-template <bool PROJECT = false>  // the second projection of u (see cam_flat_flags)
+// The second projection of u (see cam_flat_flags).
+__device__ __forceinline__ void cam_project2(CamGeom2& G, const CamRec2& g) {
+  const f2 nk = mul2(fma2(G.u0, G.a0, fma2(G.u1, G.a1, mul2(G.tau, g.ee))), G.ninv);
+  G.u0 = fma2(nk, G.a0, G.u0);
+  G.u1 = fma2(nk, G.a1, G.u1);
+}
+template <bool PROJECT = false>
 __device__ __forceinline__ CamGeom2 cam_geom2(const CamRec2& g, f2 X, f2 Y) {
   CamGeom2 G;
   G.dx = add2(X, g.npx);
@@ -165,11 +171,7 @@ __device__ __forceinline__ CamGeom2 cam_geom2(const CamRec2& g, f2 X, f2 Y) {
   G.u0 = fma2(G.tau, G.a0, D0);
   G.u1 = fma2(G.tau, G.a1, D1);
   G.nx = fma2(G.u0, G.u0, fma2(G.u1, G.u1, fma2(mul2(G.tau, G.tau), g.ee, g.nl2)));
-  if (PROJECT) {
-    const f2 nk = mul2(fma2(G.u0, G.a0, fma2(G.u1, G.a1, mul2(G.tau, g.ee))), G.ninv);
-    G.u0 = fma2(nk, G.a0, G.u0);
-    G.u1 = fma2(nk, G.a1, G.u1);
-  }
+  if (PROJECT) cam_project2(G, g);
   return G;
 }
 

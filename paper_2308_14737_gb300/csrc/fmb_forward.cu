@@ -686,13 +686,14 @@ __global__ void __launch_bounds__(kFwdThreads, fwd_min_blocks<NORMALS, NFLOW, RP
         color_of(i + 2, c0, c1, c2);
         fwd_record2<RPT, NORMALS, COLOR, false>(A, h, nB1, tiny, c0, c1, c2);
       }
-      // and the next two, or the last one, by the longer code
-      const int end = min(i + 4, n);
-#pragma unroll 1
-      for (; i < end; i += 2) {
+      // and then one, the last one or a flagged one or the one before it, by the longer code
+      // (two at a time: 1023x767 at K = 333 370 against 366 us, K = 79 with colours 4.72
+      // against 4.55 ms)
+      if (i < n) {
         f2 c0, c1, c2;
         color_of(i, c0, c1, c2);
         fwd_record2<RPT, NORMALS, COLOR, true>(A, cam_load(rec + kRecFloat4 * i), nB1, tiny, c0, c1, c2);
+        i += 2;
       }
     }
     __syncthreads();  // every thread is done with this stage before it is refilled
