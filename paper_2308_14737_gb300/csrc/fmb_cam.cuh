@@ -53,8 +53,9 @@ constexpr int kCamFlat = 1, kCamCopy = 2, kCamFlatter = 4;
 // the forward projects from a ratio of 5 on (4 % of the benchmark's Gaussians).  The
 // gradients were within the projected form's up to a ratio of 30 (L: 1.1e-5 / 1.8e-5) and
 // past it at 100 (1.2e-4 / 0.9e-5): the adjoint, whose warps hold 64 Gaussians each, projects
-// from 16 on.  Both rules cost the benchmark's scenes 0 to 0.8 % (orbit 648.6 -> 650.8 us,
-// 1023x767 at K = 333 358 -> 361).
+// from 16 on.  Both rules cost the benchmark's scenes at most 0.3 % (orbit 648.6 ->
+// 650.8 us; 1023x767 at K = 333 358 before, 357 with one flagged record at a time); a scene of
+// discs of ratio 20 14 % forward and 4 % in the adjoint.
 __device__ __forceinline__ int cam_flat_flags(float trace, float minors, float det) {
   const bool needle = !(trace * minors < 1000.f * det);
   return (needle || !(trace * trace < 14.f * minors) ? kCamFlat : 0) |
